@@ -161,7 +161,7 @@ BM_API const char *bm_status_string(int32_t status);
  *   opt: NULL for defaults.
  * The context owns its workspace (matching, levels, roots, predecessors, one
  * (column, root) queue and a second one for the next phase's roots, the
- * endpoint list: about 4*(7*n_cols + 3*n_rows) bytes),
+ * endpoint list, the rows' entry counts: about 4*(9*n_cols + 5*n_rows) bytes),
  * allocated here.  The matching starts empty.
  */
 BM_API int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t *col_ptr,
@@ -176,11 +176,13 @@ BM_API int32_t bm_upload_csr(bm_ctx *ctx, const int32_t *h_col_ptr, const int32_
 BM_API int32_t bm_set_options(bm_ctx *ctx, const bm_options *opt);
 
 /* Cheap initial matching on the GPU (the "cheap matching" initialisation of
- * Section 4): every unmatched column scans its rows in order and claims the
- * first unmatched one with an atomic compare-and-swap.  Columns are taken in
- * three passes by degree, shortest lists first (at most 32 rows: a thread
- * each; up to 2048: a warp each, longer: a block each, dealt from lists the
- * first pass builds in the context's queue).  The result is a
+ * Section 4): every unmatched column claims, with an atomic compare-and-swap,
+ * the unmatched row of its list that the fewest columns list (ties: from a
+ * position of the list that depends on the column id).  Columns are taken by
+ * degree, shortest lists first (up to 2, 8 and 32 rows: a thread each and the
+ * whole list; up to 2048: a warp each, longer: a block each, both dealt from
+ * lists the first pass builds in the context's queue and scanned up to the
+ * first step with an unmatched row).  The result is a
  * maximal matching added to the installed one; which maximal matching it is
  * depends on thread timing.  With the deterministic option the rounds of
  * proposals described there run instead (one cooperative launch; a barrier

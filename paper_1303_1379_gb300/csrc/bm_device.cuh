@@ -175,6 +175,32 @@ __device__ __forceinline__ unsigned long long globaltimer() {
     return t;
 }
 
+// A mixing of 32 bits in which every input bit reaches every output bit (two
+// rounds of xor-shift and multiplication by odd constants, a bijection).
+__device__ __forceinline__ unsigned hash32(unsigned x) {
+    x ^= x >> 16;
+    x *= 0x9e3779b1u;
+    x ^= x >> 15;
+    x *= 0x85ebca77u;
+    x ^= x >> 16;
+    return x;
+}
+
+// A bijection of [0, 2^bits) (bits <= 31) that puts neighbours far apart, in no
+// order that a stride of the input would keep: xor-shifts and odd multipliers
+// modulo 2^bits.
+__device__ __forceinline__ unsigned scatter_bits(unsigned x, int bits) {
+    const unsigned mask = (1u << bits) - 1u;
+    const int h = (bits + 1) >> 1;
+    x = (x * 0x9e3779b1u) & mask;
+    x ^= x >> h;
+    x = (x * 0x85ebca77u) & mask;
+    x ^= x >> h;
+    x = (x * 0xc2b2ae3du) & mask;
+    x ^= x >> h;
+    return x;
+}
+
 __device__ __forceinline__ void set_error(Ctl* ctl, int code) { atomicCAS(&ctl->err, 0, code); }
 
 // Range-checked build (compiled with BM_CHECKED, the library libbmatch_checked.so):

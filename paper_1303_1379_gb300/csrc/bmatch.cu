@@ -275,8 +275,10 @@ __global__ void __launch_bounds__(1024) k_release(Params p, int n_ep) {
 }
 
 // ---- input checks, greedy, fills
+// rdeg (nullable, zero before): every row's number of entries, counted on the way for
+// the cheap matching.
 __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __restrict__ cp,
-                            const int32_t* __restrict__ ri, Ctl* ctl) {
+                            const int32_t* __restrict__ ri, Ctl* ctl, int32_t* rdeg) {
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long nthr = (long long)gridDim.x * blockDim.x;
     bool bad = false;
@@ -286,6 +288,7 @@ __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __rest
     for (long long e = tid; e < nnz; e += nthr) {
         int r = __ldg(&ri[e]);
         if (r < 0 || r >= nr) bad = true;
+        else if (rdeg) atomicAdd(&rdeg[r], 1);
     }
     if (bad) bmd::set_error(ctl, BM_ERR_INVALID_CSR);
 }
@@ -354,27 +357,36 @@ __global__ void k_fill(int32_t* a, long long n, int v) {
         a[i] = v;
 }
 
-// Cheap matching: each unmatched column claims the first unmatched row of its
-// list by CAS.  A column stays unmatched only if all its rows were taken (a
-// claim is never given back), so the result is maximal.  Three launches take
-// the columns by degree, shortest lists first (a column with few rows has few
-// chances, so it chooses before the hubs, which can still find rows far down
-// their lists):
-//  * light columns (at most GREEDY_LIGHT rows): one thread each, 4 rows per
-//    step with the loads in flight together; this pass also lists the medium
-//    and heavy columns (R-MAT puts its hubs at neighbouring ids, so the later
-//    passes deal them out from these lists instead of by id);
-//  * medium columns (up to GREEDY_MEDIUM rows): one warp each, 32 x GREEDY_U
-//    rows per step;
-//  * heavy columns (R-MAT hubs reach 60,000 rows, most of them taken by then):
-//    one block each, blockDim x GREEDY_U rows per step.
-// In the cooperative scans every thread loads GREEDY_U rows and their
-// matches, the free ones are marked, and their holders try the CAS in list
-// order until one wins, so a column still takes the first row of its list
-// that was free when it looked.
+// Cheap matching: each unmatched column claims an unmatched row of its list by
+// CAS.  A column stays unmatched only if all its rows were taken (a claim is
+// never given back), so the result is maximal.  Which row and in which order
+// decides how much is left to the search, and how far its paths reach:
+//  * a column takes the free row with the fewest entries (a row that few
+//    columns list has few chances), the first of them from a position of the
+//    list that a hash of the column id gives;
+//  * tiles of 32 columns run in a scattered order, and a tile's columns in an
+//    order of its own.  Together with the rotated lists this takes every
+//    direction out of the result: when each column starts at the front of its
+//    list, or the smaller id wins each contest, a whole mesh is matched one
+//    row over and its free rows and free columns end up at opposite sides
+//    (2000 x 2000 mesh: the search then takes 100 k levels and 590 ms; with
+//    rotated lists 53 k, with scattered tiles too 44 k, with the order inside
+//    the tiles too 12 k levels and 68 ms);
+//  * the columns go by degree, shortest lists first, in launches of their own:
+//    1-2, 3-8 and 9-32 rows (one thread each, the whole list), 33-2,048 rows
+//    (one warp each, 128 rows per step) and more (one block each, 2,048 rows
+//    per step).  The first launch lists the last two kinds (R-MAT puts its
+//    hubs at neighbouring ids, so those passes deal them out from these lists
+//    instead of by id); their scans stop at the first step with a free row.
+// state[r] is the row's number of entries while it is free and GREEDY_TAKEN
+// once it is matched, so one gather per entry answers both questions; the CAS
+// is on it, and its winner stores the two matches (no launch reads another
+// column's).  R-MAT scale 21: 272 us (first free row in list order: 262 us),
+// start 578.8 k of 587.2 k pairs (530.1 k), the search 800 us (1,042 us).
 constexpr int GREEDY_LIGHT = 32;
 constexpr int GREEDY_MEDIUM = 2048;
 constexpr int GREEDY_U = 4;
+constexpr int GREEDY_TAKEN = -1;
 
 struct GreedyLists {
     int32_t* medium;  // [nc] columns of the medium pass
@@ -382,42 +394,67 @@ struct GreedyLists {
     int32_t* count;   // [2] their lengths, zero before the light pass
 };
 
+// state[r] from the matching the passes start from (rdeg may be state itself).
+__global__ void k_greedy_state(int nr, const int32_t* __restrict__ rm, const int32_t* rdeg, int32_t* state) {
+    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nr; r += gridDim.x * blockDim.x)
+        state[r] = rm[r] == -1 ? rdeg[r] : GREEDY_TAKEN;
+}
+
+// Columns of LO < degree <= HI; LISTS: also lists the columns of the later passes.
+template <int LO, int HI, bool LISTS>
 __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int32_t* __restrict__ ri,
-                               int32_t* rm, int32_t* cm, GreedyLists gl, const Ctl* ctl) {
+                               int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl, const Ctl* ctl) {
     // after an asynchronous CSR check on the same stream: an invalid CSR is not read
     if (ctl && bmd::ld_volatile(&ctl->err) != 0) return;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < nc; base += stride) {  // block-uniform
-        const int c = (int)(base + threadIdx.x);
-        int beg = 0, end = 0;
-        if (c < nc && cm[c] == -1) {
-            beg = __ldg(&cp[c]);
-            end = __ldg(&cp[c + 1]);
+    constexpr int U = HI < 4 ? HI : 4;
+    const unsigned tiles = ((unsigned)nc + 31) >> 5;
+    const int bits = tiles > 1 ? 32 - __clz(tiles - 1) : 0;  // 2^bits >= tiles
+    const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (unsigned k0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k0 < (1u << bits); k0 += nwarps) {
+        const unsigned tile = bmd::scatter_bits(k0, bits);  // warp-uniform
+        if (tile >= tiles) continue;
+        // neighbours in an order of the tile's own (a warp's atomics go by lane)
+        const unsigned th = bmd::hash32(tile);
+        const unsigned in = (((threadIdx.x & 31) * (th | 1u) + (th >> 5)) ^ (th >> 10)) & 31u;
+        const int c = (int)(tile * 32 + in);
+        if (c >= nc) continue;
+        const int beg = __ldg(&cp[c]);
+        const int deg = __ldg(&cp[c + 1]) - beg;
+        if (LISTS ? deg <= LO : (deg <= LO || deg > HI)) continue;
+        if (cm[c] != -1) continue;
+        if (LISTS) {
+            if (deg > GREEDY_MEDIUM) bmd::push(gl.heavy, 0, &gl.count[1], c);
+            else if (deg > GREEDY_LIGHT) bmd::push(gl.medium, 0, &gl.count[0], c);
+            if (deg > HI) continue;
         }
-        const int deg = end - beg;
-        if (deg > GREEDY_MEDIUM) bmd::push(gl.heavy, 0, &gl.count[1], c);
-        else if (deg > GREEDY_LIGHT) bmd::push(gl.medium, 0, &gl.count[0], c);
-        if (deg > GREEDY_LIGHT) continue;
-        bool done = false;
-        for (int e = beg; e < end && !done; e += 4) {
-            int r[4], m[4];
+        const int rot = (int)__umulhi(bmd::hash32((unsigned)c), (unsigned)deg);
+        for (;;) {
+            int best_s = 0x7fffffff, best_r = -1;
+            for (int i = 0; i < deg; i += U) {  // U rows per step with the loads in flight together
+                int r[U], st[U];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) r[u] = e + u < end ? __ldg(&ri[e + u]) : -1;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) m[u] = r[u] >= 0 ? bmd::ld_volatile(&rm[r[u]]) : 0;
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (!done && m[u] == -1 && atomicCAS(&rm[r[u]], -1, c) == -1) {
-                    cm[c] = r[u];
-                    done = true;
+                for (int u = 0; u < U; ++u) {
+                    const int k = i + u + rot;
+                    r[u] = i + u < deg ? __ldg(&ri[beg + (k < deg ? k : k - deg)]) : -1;
                 }
+#pragma unroll
+                for (int u = 0; u < U; ++u) st[u] = r[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (st[u] >= 0 && (st[u] < best_s || best_r < 0)) { best_s = st[u]; best_r = r[u]; }
+            }
+            if (best_r < 0) break;  // every row is taken
+            if (atomicCAS(&state[best_r], best_s, GREEDY_TAKEN) == best_s) {
+                rm[best_r] = c;
+                cm[c] = best_r;
+                break;
             }
         }
     }
 }
 
-__global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri, int32_t* rm,
-                                int32_t* cm, GreedyLists gl, const Ctl* ctl) {
+__global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri, int32_t* state,
+                                int32_t* rm, int32_t* cm, GreedyLists gl, const Ctl* ctl) {
     if (ctl && bmd::ld_volatile(&ctl->err) != 0) return;
     const int lane = threadIdx.x & 31;
     const int n = gl.count[0];
@@ -428,35 +465,42 @@ __global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* _
         const int hb = __ldg(&cp[hc]), he = __ldg(&cp[hc + 1]);
         bool done = false;
         for (int e0 = hb; e0 < he && !done; e0 += 32 * GREEDY_U) {  // warp-uniform
-            int r[GREEDY_U], m[GREEDY_U];
+            int r[GREEDY_U], st[GREEDY_U];
 #pragma unroll
             for (int u = 0; u < GREEDY_U; ++u) {
                 const int e = e0 + u * 32 + lane;
                 r[u] = e < he ? __ldg(&ri[e]) : -1;
             }
 #pragma unroll
-            for (int u = 0; u < GREEDY_U; ++u) m[u] = r[u] >= 0 ? bmd::ld_volatile(&rm[r[u]]) : 0;
+            for (int u = 0; u < GREEDY_U; ++u) st[u] = r[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
+            while (!done) {  // warp-uniform: the window's free row with the fewest entries
+                int best_s = 0x7fffffff, best_u = -1, best_r = -1;
 #pragma unroll
-            for (int u = 0; u < GREEDY_U; ++u) {
-                unsigned free_lanes = __ballot_sync(bmd::FULL, m[u] == -1);
-                while (free_lanes && !done) {  // warp-uniform: lowest list position first
-                    const int l = __ffs(free_lanes) - 1;
-                    free_lanes &= free_lanes - 1;
-                    int won = 0;
-                    if (lane == l) won = atomicCAS(&rm[r[u]], -1, hc) == -1;
-                    won = __shfl_sync(bmd::FULL, won, l);
+                for (int u = 0; u < GREEDY_U; ++u)
+                    if (st[u] >= 0 && (st[u] < best_s || best_u < 0)) { best_s = st[u]; best_u = u; best_r = r[u]; }
+                if (!__any_sync(bmd::FULL, best_u >= 0)) break;  // none left: the next window
+                const int least = __reduce_min_sync(bmd::FULL, best_u >= 0 ? best_s : 0x7fffffff);
+                const int l = __ffs(__ballot_sync(bmd::FULL, best_u >= 0 && best_s == least)) - 1;
+                int won = 0;
+                if (lane == l) {
+                    won = atomicCAS(&state[best_r], best_s, GREEDY_TAKEN) == best_s;
                     if (won) {
-                        if (lane == l) cm[hc] = r[u];
-                        done = true;
+                        rm[best_r] = hc;
+                        cm[hc] = best_r;
                     }
+#pragma unroll
+                    for (int u = 0; u < GREEDY_U; ++u)
+                        if (u == best_u) st[u] = GREEDY_TAKEN;
                 }
+                done = __shfl_sync(bmd::FULL, won, l) != 0;
             }
         }
     }
 }
 
 __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri,
-                                                       int32_t* rm, int32_t* cm, GreedyLists gl, const Ctl* ctl) {
+                                                       int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl,
+                                                       const Ctl* ctl) {
     if (ctl && bmd::ld_volatile(&ctl->err) != 0) return;
     __shared__ int s_pos, s_done;
     const int T = blockDim.x, t = threadIdx.x;
@@ -474,12 +518,12 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
                 r[u] = e < he ? __ldg(&ri[e]) : -1;
             }
 #pragma unroll
-            for (int u = 0; u < GREEDY_U; ++u) m[u] = r[u] >= 0 ? bmd::ld_volatile(&rm[r[u]]) : 0;
+            for (int u = 0; u < GREEDY_U; ++u) m[u] = r[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
             // window position of this thread's first free row (list order: u major, thread minor)
             int pos = 0x7fffffff;
 #pragma unroll
             for (int u = GREEDY_U - 1; u >= 0; --u)
-                if (m[u] == -1) pos = u * T + t;
+                if (m[u] >= 0) pos = u * T + t;
             if (t == 0) s_pos = 0x7fffffff;
             __syncthreads();
             if (pos != 0x7fffffff) atomicMin(&s_pos, pos);
@@ -490,11 +534,12 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
                 __syncthreads();  // every thread has read s_pos
                 if (t == mypos % T) {
                     const int u = mypos / T;
-                    int rr = -1;
+                    int rr = -1, seen = 0;
 #pragma unroll
                     for (int v = 0; v < GREEDY_U; ++v)
-                        if (v == u) rr = r[v];
-                    if (atomicCAS(&rm[rr], -1, hc) == -1) {
+                        if (v == u) { rr = r[v]; seen = m[v]; }
+                    if (atomicCAS(&state[rr], seen, GREEDY_TAKEN) == seen) {
+                        rm[rr] = hc;
                         cm[hc] = rr;
                         s_done = 1;
                     }
@@ -505,7 +550,7 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
                     int next = 0x7fffffff;
 #pragma unroll
                     for (int u = GREEDY_U - 1; u >= 0; --u)
-                        if (m[u] == -1 && u * T + t > mypos) next = u * T + t;
+                        if (m[u] >= 0 && u * T + t > mypos) next = u * T + t;
                     if (next != 0x7fffffff) atomicMin(&s_pos, next);
                 }
                 __syncthreads();
@@ -516,15 +561,21 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
     }
 }
 
-// The cheap matching (Section 4) on the device: light, medium and heavy
-// columns in this order.  `lists` is scratch of 2 x nc int32 (the context's
-// queue, free before a match) and `count` two int32 cleared beforehand.
-void launch_greedy(int nc, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, const Ctl* ctl,
-                   int32_t* lists, int32_t* count, int grid, int block, cudaStream_t st) {
+// The cheap matching (Section 4) on the device: columns by degree, shortest
+// lists first.  `rdeg` holds the rows' entry counts, `state` is scratch of nr
+// int32 (it may be rdeg, whose counts are then lost), `lists` of 2 x nc int32
+// (the context's queue, free before a match) and `count` two int32 cleared
+// beforehand.
+void launch_greedy(int nr, int nc, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, const Ctl* ctl,
+                   const int32_t* rdeg, int32_t* state, int32_t* lists, int32_t* count, int grid, int block,
+                   cudaStream_t st) {
     const GreedyLists gl{lists, lists + nc, count};
-    k_greedy_light<<<grid, block, 0, st>>>(nc, cp, ri, rm, cm, gl, ctl);
-    k_greedy_medium<<<grid, block, 0, st>>>(cp, ri, rm, cm, gl, ctl);
-    k_greedy_heavy<<<grid, block, 0, st>>>(cp, ri, rm, cm, gl, ctl);
+    k_greedy_state<<<grid, block, 0, st>>>(nr, rm, rdeg, state);
+    k_greedy_light<0, 2, true><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    k_greedy_medium<<<grid, block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
+    k_greedy_heavy<<<grid, block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
 }
 
 // The cheap matching of the deterministic option over the whole GPU (one
@@ -668,6 +719,7 @@ struct bm_ctx {
     int2* queue2 = nullptr;  // roots of the next phase (one-endpoint GPUBFS-WR)
     int32_t* endpoints = nullptr;
     int32_t* rvis = nullptr;     // per-row claim stamps of the persistent kernel
+    int32_t* rdeg = nullptr;     // per-row number of entries, counted by the CSR check (cheap matching)
     int2* crec = nullptr;        // per-column (parent column, matched row) of the last search
     long long stamp_next = 0;    // every stamp in rvis is below stamp_next + 1
     int32_t* profile = nullptr;  // kProfileCap phases x 4
@@ -785,7 +837,9 @@ Params make_params(bm_ctx* ctx, bool bfs_only) {
 int32_t validate_csr_async(bm_ctx* ctx) {
     const long long work = ctx->nnz > ctx->nc ? ctx->nnz : (long long)ctx->nc + 1;
     const int g = grid_for(ctx, (int)(work < (1 << 30) ? work : (1 << 30)));
-    k_check_csr<<<g, ctx->block, 0, ctx->stream>>>(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->ctl);
+    if (ctx->nr) BM_CUDA(ctx, cudaMemsetAsync(ctx->rdeg, 0, 4 * (size_t)ctx->nr, ctx->stream));
+    k_check_csr<<<g, ctx->block, 0, ctx->stream>>>(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->ctl,
+                                                   ctx->rdeg);
     BM_CUDA(ctx, cudaGetLastError());
     return BM_OK;
 }
@@ -1052,7 +1106,7 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
     if (!coop) { delete ctx; return BM_ERR_UNSUPPORTED; }
 
     // arena: [ctl][rmatch nr][cmatch nc][level nc][root nc][pred nr][queue nc][queue2 nc][endpoints nr]
-    //        [rvis nr][crec nc][profile][csr?]
+    //        [rvis nr][crec nc][rdeg nr][profile][csr?]
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
     const size_t nr1 = (size_t)(n_rows ? n_rows : 1), nc1 = (size_t)(n_cols ? n_cols : 1);
     size_t off_ctl = 0;
@@ -1066,7 +1120,8 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
     size_t off_ep = off_q2 + al(8 * nc1);
     size_t off_rv = off_ep + al(4 * nr1);
     size_t off_cr = off_rv + al(4 * nr1);
-    size_t off_pf = off_cr + al(8 * nc1);
+    size_t off_rd = off_cr + al(8 * nc1);
+    size_t off_pf = off_rd + al(4 * nr1);
     size_t off_cp = off_pf + al(4 * 4 * (size_t)kProfileCap);
     size_t total = off_cp;
     const bool own = (col_ptr == nullptr);
@@ -1098,6 +1153,7 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
     ctx->endpoints = (int32_t*)(a + off_ep);
     ctx->rvis = (int32_t*)(a + off_rv);
     ctx->crec = (int2*)(a + off_cr);
+    ctx->rdeg = (int32_t*)(a + off_rd);
     ctx->profile = (int32_t*)(a + off_pf);
     if (own) {
         ctx->owns_csr = true;
@@ -1177,8 +1233,8 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
         BM_CUDA(ctx, cudaGetLastError());
     } else if (ctx->nc) {
-        launch_greedy(ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, nullptr, (int32_t*)ctx->queue,
-                      &ctx->ctl->qcnt[0], grid_for(ctx, ctx->nc), ctx->block, st);
+        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, nullptr, ctx->rdeg,
+                      ctx->endpoints, (int32_t*)ctx->queue, &ctx->ctl->qcnt[0], grid_for(ctx, ctx->nc), ctx->block, st);
         BM_CUDA(ctx, cudaGetLastError());
         k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
         BM_CUDA(ctx, cudaGetLastError());
@@ -1497,7 +1553,7 @@ extern "C" int32_t bm_match_noalloc(int32_t n_rows, int32_t n_cols, int64_t nnz,
     int g = (int)((work + d.block - 1) / d.block);
     if (g > threads) g = threads;
     if (g < 1) g = 1;
-    k_check_csr<<<g, d.block, 0, st>>>(n_rows, n_cols, nnz, col_ptr, row_idx, ctl);
+    k_check_csr<<<g, d.block, 0, st>>>(n_rows, n_cols, nnz, col_ptr, row_idx, ctl, nullptr);
     const int n_max = n_rows > n_cols ? n_rows : n_cols;
     int g2 = (n_max + d.block - 1) / d.block;
     if (g2 > threads) g2 = threads;
@@ -1574,8 +1630,11 @@ int32_t bmi::enqueue_match(bmd::Params p, long long nnz, bool wr, int greedy, cu
     };
     const size_t nr = (size_t)p.nr, nc = (size_t)p.nc;
     if (cudaMemsetAsync(p.ctl, 0, sizeof(Ctl), st) != cudaSuccess) { (void)cudaGetLastError(); return BM_ERR_CUDA; }
+    // the cheap matching's entry counts go where the search keeps its predecessors
+    int32_t* const rdeg = greedy && !p.dkey ? p.pred : nullptr;
+    if (rdeg && nr && cudaMemsetAsync(rdeg, 0, 4 * nr, st) != cudaSuccess) { (void)cudaGetLastError(); return BM_ERR_CUDA; }
     k_check_csr<<<grid_of(nnz > p.nc ? nnz : (long long)p.nc + 1), B, 0, st>>>(p.nr, p.nc, nnz, p.col_ptr,
-                                                                               p.row_idx, p.ctl);
+                                                                               p.row_idx, p.ctl, rdeg);
     if ((nr && (cudaMemsetAsync(p.rmatch, 0xff, 4 * nr, st) != cudaSuccess ||
                 cudaMemsetAsync(p.rvis, 0, 4 * nr, st) != cudaSuccess)) ||
         (nc && cudaMemsetAsync(p.cmatch, 0xff, 4 * nc, st) != cudaSuccess)) {
@@ -1604,8 +1663,8 @@ int32_t bmi::enqueue_match(bmd::Params p, long long nnz, bool wr, int greedy, cu
     } else if (greedy) {
         // the cheap matching counts its lists in the control block's first two queue
         // counters, which the matching kernel needs at zero
-        launch_greedy(p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, (int32_t*)p.queue, &p.ctl->qcnt[0],
-                      grid_of(p.nc), B, st);
+        launch_greedy(p.nr, p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, rdeg, rdeg, (int32_t*)p.queue,
+                      &p.ctl->qcnt[0], grid_of(p.nc), B, st);
         if (cudaMemsetAsync(&p.ctl->qcnt[0], 0, 2 * sizeof(int32_t), st) != cudaSuccess) {
             (void)cudaGetLastError();
             return BM_ERR_CUDA;
