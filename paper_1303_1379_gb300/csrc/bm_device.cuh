@@ -492,6 +492,46 @@ __device__ __forceinline__ void step_next_roots(const Params& p, const int2* q, 
     flush_block(p, q_next, sm, 0, slot);  // a full buffer spills to global appends meanwhile
 }
 
+// Between phases while search trees are carried over (k_match): the entries of
+// trees whose root took no endpoint stay in the forest and are appended to the
+// other queue buffer (only the roots, when keep_trees is off); the columns of
+// the other trees go back to "unvisited", and so do the rows they were reached
+// through (rv_free: a stamp below the phases').  A root is served when its
+// level slot is not L0: -(row), or L0 - 1 once its own entry was reset here.
+// Runs beside Alternate's walks, like step_next_roots.
+__device__ __forceinline__ void step_carry(const Params& p, const int2* q, int tail, int2* q_next, int slot,
+                                           bool keep_trees, int rv_free, Smem& sm) {
+    const int T = blockDim.x;
+    const int per = T <= QBUF / 4 ? 4 : QBUF / T;  // entries per thread per pass: at most QBUF a block
+    for (int base = blockIdx.x * per * T; base < tail; base += gridDim.x * per * T) {  // block-uniform
+        int2 e[4];
+        int lv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = base + u * T + (int)threadIdx.x;
+            e[u] = (u < per && i < tail) ? __ldcg(&q[i]) : make_int2(-1, -1);
+            if (e[u].x >= 0 && (!idx_ok(p, e[u].x, p.nc) || !idx_ok(p, e[u].y, p.nc))) e[u].x = -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) lv[u] = e[u].x >= 0 ? __ldcg(&p.level[e[u].y]) : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (e[u].x < 0) continue;
+            if (lv[u] == L0 && (keep_trees || e[u].x == e[u].y)) {
+                push_block(p, q_next, sm, 0, slot, e[u]);
+            } else {
+                __stcg(&p.level[e[u].x], L0 - 1);
+                __stcg(&p.root[e[u].x], -1);
+                if (e[u].x != e[u].y) {
+                    const int r = __ldcg(&p.crec[e[u].x]).y;
+                    if (idx_ok(p, r, p.nr)) __stcg(&p.rvis[r], rv_free);
+                }
+            }
+        }
+        flush_block(p, q_next, sm, 0, slot);
+    }
+}
+
 // ------------------------------------------------------------------ BFS level
 // Loads tile entries [qb + first, qb + first + tw) of the queue (one per
 // thread; threads >= tw idle) and lays the tile's adjacency out in shared
@@ -1276,14 +1316,17 @@ __device__ __forceinline__ void step_alternate(const Params& p, int n_ep, int ca
 // follows the per-column records written by the BFS, one 8-byte load per
 // step: column c on the path has (parent column, its old matched row); c is
 // rematched to the row below it, and the walk continues from the old row's
-// parent.  The root's record is (-1, -1).
-__device__ __forceinline__ void step_alternate_disjoint(const Params& p, int n_ep, int cap) {
+// parent.  The root's record is (-1, -1).  rv_free (>= 0: trees are carried
+// over): the endpoint row, matched from here on, is marked "unvisited" (a level
+// that claims through the row stamps may have stamped it while it was free).
+__device__ __forceinline__ void step_alternate_disjoint(const Params& p, int n_ep, int cap, int rv_free = -1) {
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthr = gridDim.x * blockDim.x;
     unsigned steps_done = 0;
     for (int i = tid; i < n_ep; i += nthr) {
         int r = __ldcg(&p.endpoints[i]);
         if (!idx_ok(p, r, p.nr)) continue;
+        if (rv_free >= 0) __stcg(&p.rvis[r], rv_free);
         int c = __ldcg(&p.pred[r]);
         int steps = 0;
         for (;;) {

@@ -43,6 +43,28 @@ struct LeaderStats {
     int levels, first_ep, last_ep;
 };
 
+// Carried search trees (the default mode: APFB, GPUBFS-WR, one endpoint per root; a
+// context's launches).  After a phase only the trees that took an endpoint give their
+// columns back; the others stay, and the next phase starts from all their columns, so
+// that it searches what became free instead of building the same forest again.  A phase
+// that searches on from every kept column and finds neither a free row nor a free-to-claim
+// column has shown the forest closed, as a search from the roots would.  And since a
+// phase that ends early loses nothing, one that has found endpoints ends once its levels
+// are narrow (a few columns a level against the forest: each level is a round trip of the
+// whole grid, and starting the next phase costs about two).
+// Long augmenting paths do not gain from it: a carried tree's paths are not the shortest.
+// So a search that needs many phases stops cutting them short after CUT_PHASES and starts
+// from its roots again after CARRY_PHASES.  One GB300, search alone, before -> after
+// (phases / levels): 300 k uniform graph 776 -> 465 us (5 / 130 -> 8 / 44); R-MAT 1 M
+// 521 -> 418 us (4 / 44 -> 5 / 22); R-MAT scale 21 786 -> 658 us; 2000 x 2000 mesh 66 -> 57 ms
+// (13 / 11.4 k -> 20 / 9.5 k; 62 ms cut for 6 phases only, 71 ms rebuilt after 10); the mesh
+// from the one-sided start of a first-free-row matching 210 -> 201 ms (417 ms if carried to
+// the end).  CUT_MIN 3 to 7 and no ratio are within 5% on the random graphs.
+constexpr int CARRY_PHASES = 20;
+constexpr int CUT_PHASES = 10;
+constexpr int CUT_MIN = 5, CUT_MAX = 24;  // levels of a phase after which it may be cut
+constexpr int CUT_RATIO = 16;             // ... if the next has at most 1 / CUT_RATIO of the forest's columns
+
 // One launch per match: Algorithm 1 with both loops on the device.  RV: small
 // BFS levels claim columns through the row stamps p.rvis (a context's
 // launches); without it every level claims through the column levels (the
@@ -71,7 +93,9 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
     int card = 0;
     int status = 0;
     int n_roots = 0;
+    int n_front = 0;  // entries of the phase's first queue segment: its roots, and the trees carried over
     int iso_free = 0;
+    bool carry = RV && !DET && incr && p.mode == 0;  // trees are carried over to the next phase (see below)
     int no_roots = 0;  // the loop ended because no column was left to search from
     if (ld_volatile(&ctl->err) != 0) goto out;  // input validation failed before launch
     {
@@ -87,7 +111,7 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
         }
         step_init<WR>(p, qcur, s % 3, cnt, sm);
         if (!grid_sync(ctl, bid, p.wait_ns, deadline, sm, &ctl->ecnt[s % 3], &ctl->icnt[s % 3])) goto out;
-        n_roots = sm.bc_a;       // unmatched columns with rows: the first queue segment
+        n_roots = n_front = sm.bc_a;  // unmatched columns with rows: the first queue segment
         card = p.nc - sm.bc_c;   // all unmatched columns
         iso_free = sm.bc_d;      // unmatched columns without rows (never matchable)
         if (leader) ctl->initial_card = card;
@@ -102,9 +126,12 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
         // the phase's endpoint counter (incremental mode: two, alternating by phase,
         // each cleared during the phase before it uses it)
         int32_t* const epc = (incr && (phases & 1) == 0) ? &ctl->ep_alt : &ctl->ep_phase;
+        const bool graft = carry;  // this phase's
+        const int stamp = p.stamp_base + (graft ? 1 : phases);  // carried rows keep their stamp
 
         // ---- BFS, level by level (Algorithm 1 inner loop)
-        int qb = 0, qe = n_roots, lvl = L0, tail = n_roots;
+        int qb = 0, qe = n_front, lvl = L0, tail = n_front;
+        bool any_ep = false;
         if (leader) { ls.levels = 0; ls.first_ep = 0; ls.last_ep = 0; ls.roots_total += n_roots; }
         for (;;) {
             const int s2 = step++;
@@ -113,7 +140,7 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
                 if (DET) ctl->dcnt[(s2 + 1) % 3] = 0;
             }
             if constexpr (DET) step_expand_det(p, qcur, qb, qe, lvl, s2 % 3, cnt, sm);
-            else step_expand<WR, RV, true>(p, qcur, qb, qe, lvl, s2 % 3, cnt, sm, p.stamp_base + phases, epc);
+            else step_expand<WR, RV, true>(p, qcur, qb, qe, lvl, s2 % 3, cnt, sm, stamp, epc);
             if (!grid_sync(ctl, bid, p.wait_ns, deadline, sm, DET ? &ctl->dcnt[s2 % 3] : nullptr)) goto out;
             const int nq = sm.bc_a;           // columns inserted at this level
             const bool found = sm.bc_b > 0;   // some block claimed an endpoint (DET: received an offer)
@@ -137,6 +164,11 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
             tail = qe + nq;
             if (nq == 0) break;              // no vertex inserted
             if (p.mode == 1 && found) break;  // APsB: stop at the first level with a path
+            any_ep |= found;
+            // what is left of a carried search is narrow: augment, and search on from its trees
+            if (graft && any_ep && phases <= CUT_PHASES && lvl - L0 + 1 >= CUT_MIN && lvl - L0 + 1 <= CUT_MAX &&
+                (long long)nq * CUT_RATIO <= tail)
+                break;
             qb = qe;
             qe += nq;
             ++lvl;
@@ -175,8 +207,10 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
                 if (DET) ctl->dcnt[(s3 + 1) % 3] = 0;
                 *(epc == &ctl->ep_phase ? &ctl->ep_alt : &ctl->ep_phase) = 0;  // the next phase's counter
             }
-            step_alternate_disjoint(p, n_ep, tail + 2);
-            step_next_roots<WR, DET, true>(p, qcur, n_roots, tail, qnext, s3 % 3, sm);
+            step_alternate_disjoint(p, n_ep, tail + 2, DET ? -1 : p.stamp_base);
+            if (phases >= CARRY_PHASES) carry = false;
+            if (graft) step_carry(p, qcur, tail, qnext, s3 % 3, carry, p.stamp_base, sm);
+            else step_next_roots<WR, DET, true>(p, qcur, n_roots, tail, qnext, s3 % 3, sm);
         } else {
             step_alternate(p, n_ep, tail + 2, cnt);
             if (!grid_sync(ctl, bid, p.wait_ns, deadline, sm, nullptr)) goto out;
@@ -192,7 +226,8 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
         if (incr) {
             // ---- next phase's roots: the unmatched ones among this phase's roots
             if (!grid_sync(ctl, bid, p.wait_ns, deadline, sm, nullptr)) goto out;
-            n_roots = sm.bc_a;
+            n_front = sm.bc_a;
+            n_roots = graft ? n_roots - n_ep : n_front;  // every endpoint serves one root
 #ifdef BM_CHECKED
             step_check_matching(p);
             if (!grid_sync(ctl, bid, p.wait_ns, deadline, sm, &ctl->err)) goto out;
@@ -213,7 +248,7 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
             }
             step_init<WR>(p, qcur, s % 3, cnt, sm);
             if (!grid_sync(ctl, bid, p.wait_ns, deadline, sm, &ctl->ecnt[s % 3])) goto out;
-            n_roots = sm.bc_a;
+            n_roots = n_front = sm.bc_a;
             card = p.nc - sm.bc_c;
 #ifdef BM_CHECKED
             step_check_matching(p);
