@@ -21,7 +21,7 @@ INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "libbmatch.so")
 LIB_CHECKED = os.path.join(HERE, "libbmatch_checked.so")
 SOURCES = [os.path.join(CSRC, f) for f in ("bmatch.cu", "bm_batch.cu", "bm_server.cu")]
-DEPENDS = SOURCES + [os.path.join(CSRC, f) for f in ("bm_device.cuh", "bm_internal.h", "bm_pool.h")] + \
+DEPENDS = SOURCES + [os.path.join(CSRC, f) for f in ("bm_device.cuh", "bm_internal.h", "bm_pool.h", "bm_solo.cuh")] + \
     [os.path.join(INCLUDE, "bmatch.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

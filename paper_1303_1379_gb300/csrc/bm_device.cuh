@@ -57,6 +57,28 @@ constexpr int HUB_DEG = 256;  // warp-level expansion: columns of more edges are
 constexpr int HUB_MAX = 16;   // ... at most this many per level (the rest stay with their warp)
 constexpr int RV_MAX_Q = 32768;  // largest level (columns) that claims through row stamps
 
+// Carried search trees (the default mode: APFB, GPUBFS-WR, one endpoint per root; a
+// context's launches).  After a phase only the trees that took an endpoint give their
+// columns back; the others stay, and the next phase starts from all their columns, so
+// that it searches what became free instead of building the same forest again.  A phase
+// that searches on from every kept column and finds neither a free row nor a free-to-claim
+// column has shown the forest closed, as a search from the roots would.  And since a
+// phase that ends early loses nothing, one that has found endpoints ends once its levels
+// are narrow (a few columns a level against the forest: each level is a round trip of the
+// whole grid, and starting the next phase costs about two).
+// Long augmenting paths do not gain from it: a carried tree's paths are not the shortest.
+// So a search that needs many phases stops cutting them short after CUT_PHASES and starts
+// from its roots again after CARRY_PHASES.  One GB300, search alone, before -> after
+// (phases / levels): 300 k uniform graph 776 -> 465 us (5 / 130 -> 8 / 44); R-MAT 1 M
+// 521 -> 418 us (4 / 44 -> 5 / 22); R-MAT scale 21 786 -> 658 us; 2000 x 2000 mesh 66 -> 57 ms
+// (13 / 11.4 k -> 20 / 9.5 k; 62 ms cut for 6 phases only, 71 ms rebuilt after 10); the mesh
+// from the one-sided start of a first-free-row matching 210 -> 201 ms (417 ms if carried to
+// the end).  CUT_MIN 3 to 7 and no ratio are within 5% on the random graphs.
+constexpr int CARRY_PHASES = 20;
+constexpr int CUT_PHASES = 10;
+constexpr int CUT_MIN = 5, CUT_MAX = 24;  // levels of a phase after which it may be cut
+constexpr int CUT_RATIO = 16;             // ... if the next has at most 1 / CUT_RATIO of the forest's columns
+
 // Control block in device memory, cleared before every launch.  Per-step
 // counters rotate over three slots: step s appends to slot s % 3 and clears
 // slot (s + 1) % 3, which nobody reads during step s (it was last read right
@@ -373,6 +395,79 @@ __device__ __forceinline__ void add_to_counter(long long* dst, unsigned v) {
 #pragma unroll
     for (int s = 16; s >= 1; s >>= 1) a += __shfl_down_sync(FULL, a, s);
     if ((threadIdx.x & 31) == 0 && a) atomicAdd((unsigned long long*)dst, a);
+}
+
+// ------------------------------------------------------------------ cheap matching
+constexpr int GREEDY_LIGHT = 32;     // columns of at most this many rows: a thread each
+constexpr int GREEDY_MEDIUM = 2048;  // ... and this many: a warp each
+constexpr int GREEDY_U = 4;          // rows per thread and step of the cooperative scans
+constexpr int GREEDY_TAKEN = -1;     // state of a matched row; a free row's is its number of entries
+
+// The free row with the fewest entries of a list of deg rows, the first such
+// from position rot on (wrapping); U rows per step with the loads in flight
+// together.  Returns the row (-1: none is free) and the state it was seen with.
+template <int U, class State>
+__device__ __forceinline__ int greedy_pick(const int32_t* __restrict__ list, int deg, int rot, State state, int& seen) {
+    int best_s = 0x7fffffff, best_r = -1;
+    for (int i = 0; i < deg; i += U) {
+        int r[U], st[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int k = i + u + rot;
+            r[u] = i + u < deg ? __ldg(&list[k < deg ? k : k - deg]) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) st[u] = r[u] >= 0 ? state(r[u]) : GREEDY_TAKEN;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (st[u] >= 0 && (st[u] < best_s || best_r < 0)) { best_s = st[u]; best_r = r[u]; }
+    }
+    seen = best_s;
+    return best_r;
+}
+
+// A warp takes a free row of a list of n rows: 32 x GREEDY_U rows per step, of
+// the first step with a free row the one with the fewest entries that no one
+// takes meanwhile.  Returns the row (every lane; -1: none).
+template <class State, class Take>
+__device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int n, State state_of, Take take) {
+    const int lane = threadIdx.x & 31;
+    for (int e0 = 0; e0 < n; e0 += 32 * GREEDY_U) {  // warp-uniform
+        int r[GREEDY_U], st[GREEDY_U];
+#pragma unroll
+        for (int u = 0; u < GREEDY_U; ++u) {
+            const int e = e0 + u * 32 + lane;
+            r[u] = e < n ? __ldg(&list[e]) : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < GREEDY_U; ++u) st[u] = r[u] >= 0 ? state_of(r[u]) : GREEDY_TAKEN;
+        for (;;) {  // warp-uniform: the window's free row with the fewest entries
+            int best_s = 0x7fffffff, best_u = -1, best_r = -1;
+#pragma unroll
+            for (int u = 0; u < GREEDY_U; ++u)
+                if (st[u] >= 0 && (st[u] < best_s || best_u < 0)) { best_s = st[u]; best_u = u; best_r = r[u]; }
+            if (!__any_sync(FULL, best_u >= 0)) break;  // none left: the next window
+            const int least = __reduce_min_sync(FULL, best_u >= 0 ? best_s : 0x7fffffff);
+            const int l = __ffs(__ballot_sync(FULL, best_u >= 0 && best_s == least)) - 1;
+            int won = -1;
+            if (lane == l) {
+                if (take(best_r, best_s)) won = best_r;
+#pragma unroll
+                for (int u = 0; u < GREEDY_U; ++u)
+                    if (u == best_u) st[u] = GREEDY_TAKEN;
+            }
+            won = __shfl_sync(FULL, won, l);
+            if (won >= 0) return won;
+        }
+    }
+    return -1;
+}
+
+// The column that a lane of a tile of 32 takes: neighbours in an order of the
+// tile's own (a warp's atomics go by lane).
+__device__ __forceinline__ int scatter_lane(unsigned tile, int lane) {
+    const unsigned th = hash32(tile);
+    return (int)(tile * 32 + ((((unsigned)lane * (th | 1u) + (th >> 5)) ^ (th >> 10)) & 31u));
 }
 
 // ------------------------------------------------------------------ InitBfsArray

@@ -18,6 +18,7 @@
 
 #include "bm_device.cuh"
 #include "bm_internal.h"
+#include "bm_solo.cuh"
 #include "bmatch.h"
 
 using bmd::Counters;
@@ -42,28 +43,6 @@ struct LeaderStats {
     long long levels_total, levels_max, eps_total, ins_total, roots_total;
     int levels, first_ep, last_ep;
 };
-
-// Carried search trees (the default mode: APFB, GPUBFS-WR, one endpoint per root; a
-// context's launches).  After a phase only the trees that took an endpoint give their
-// columns back; the others stay, and the next phase starts from all their columns, so
-// that it searches what became free instead of building the same forest again.  A phase
-// that searches on from every kept column and finds neither a free row nor a free-to-claim
-// column has shown the forest closed, as a search from the roots would.  And since a
-// phase that ends early loses nothing, one that has found endpoints ends once its levels
-// are narrow (a few columns a level against the forest: each level is a round trip of the
-// whole grid, and starting the next phase costs about two).
-// Long augmenting paths do not gain from it: a carried tree's paths are not the shortest.
-// So a search that needs many phases stops cutting them short after CUT_PHASES and starts
-// from its roots again after CARRY_PHASES.  One GB300, search alone, before -> after
-// (phases / levels): 300 k uniform graph 776 -> 465 us (5 / 130 -> 8 / 44); R-MAT 1 M
-// 521 -> 418 us (4 / 44 -> 5 / 22); R-MAT scale 21 786 -> 658 us; 2000 x 2000 mesh 66 -> 57 ms
-// (13 / 11.4 k -> 20 / 9.5 k; 62 ms cut for 6 phases only, 71 ms rebuilt after 10); the mesh
-// from the one-sided start of a first-free-row matching 210 -> 201 ms (417 ms if carried to
-// the end).  CUT_MIN 3 to 7 and no ratio are within 5% on the random graphs.
-constexpr int CARRY_PHASES = 20;
-constexpr int CUT_PHASES = 10;
-constexpr int CUT_MIN = 5, CUT_MAX = 24;  // levels of a phase after which it may be cut
-constexpr int CUT_RATIO = 16;             // ... if the next has at most 1 / CUT_RATIO of the forest's columns
 
 // One launch per match: Algorithm 1 with both loops on the device.  RV: small
 // BFS levels claim columns through the row stamps p.rvis (a context's
@@ -166,7 +145,7 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
             if (p.mode == 1 && found) break;  // APsB: stop at the first level with a path
             any_ep |= found;
             // what is left of a carried search is narrow: augment, and search on from its trees
-            if (graft && any_ep && phases <= CUT_PHASES && lvl - L0 + 1 >= CUT_MIN && lvl - L0 + 1 <= CUT_MAX &&
+            if (graft && any_ep && phases <= bmd::CUT_PHASES && lvl - L0 + 1 >= CUT_MIN && lvl - L0 + 1 <= CUT_MAX &&
                 (long long)nq * CUT_RATIO <= tail)
                 break;
             qb = qe;
@@ -418,10 +397,10 @@ __global__ void k_fill(int32_t* a, long long n, int v) {
 // is on it, and its winner stores the two matches (no launch reads another
 // column's).  R-MAT scale 21: 272 us (first free row in list order: 262 us),
 // start 578.8 k of 587.2 k pairs (530.1 k), the search 800 us (1,042 us).
-constexpr int GREEDY_LIGHT = 32;
-constexpr int GREEDY_MEDIUM = 2048;
-constexpr int GREEDY_U = 4;
-constexpr int GREEDY_TAKEN = -1;
+using bmd::GREEDY_LIGHT;
+using bmd::GREEDY_MEDIUM;
+using bmd::GREEDY_TAKEN;
+using bmd::GREEDY_U;
 
 struct GreedyLists {
     int32_t* medium;  // [nc] columns of the medium pass
@@ -448,10 +427,7 @@ __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int
     for (unsigned k0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k0 < (1u << bits); k0 += nwarps) {
         const unsigned tile = bmd::scatter_bits(k0, bits);  // warp-uniform
         if (tile >= tiles) continue;
-        // neighbours in an order of the tile's own (a warp's atomics go by lane)
-        const unsigned th = bmd::hash32(tile);
-        const unsigned in = (((threadIdx.x & 31) * (th | 1u) + (th >> 5)) ^ (th >> 10)) & 31u;
-        const int c = (int)(tile * 32 + in);
+        const int c = bmd::scatter_lane(tile, threadIdx.x & 31);
         if (c >= nc) continue;
         const int beg = __ldg(&cp[c]);
         const int deg = __ldg(&cp[c + 1]) - beg;
@@ -464,24 +440,12 @@ __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int
         }
         const int rot = (int)__umulhi(bmd::hash32((unsigned)c), (unsigned)deg);
         for (;;) {
-            int best_s = 0x7fffffff, best_r = -1;
-            for (int i = 0; i < deg; i += U) {  // U rows per step with the loads in flight together
-                int r[U], st[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int k = i + u + rot;
-                    r[u] = i + u < deg ? __ldg(&ri[beg + (k < deg ? k : k - deg)]) : -1;
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) st[u] = r[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (st[u] >= 0 && (st[u] < best_s || best_r < 0)) { best_s = st[u]; best_r = r[u]; }
-            }
-            if (best_r < 0) break;  // every row is taken
-            if (atomicCAS(&state[best_r], best_s, GREEDY_TAKEN) == best_s) {
-                rm[best_r] = c;
-                cm[c] = best_r;
+            int seen;
+            const int r = bmd::greedy_pick<U>(ri + beg, deg, rot, [&](int k) { return bmd::ld_volatile(&state[k]); }, seen);
+            if (r < 0) break;  // every row is taken
+            if (atomicCAS(&state[r], seen, GREEDY_TAKEN) == seen) {
+                rm[r] = c;
+                cm[c] = r;
                 break;
             }
         }
@@ -498,37 +462,12 @@ __global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* _
     for (long long k = warp; k < n; k += nwarps) {  // warp-uniform
         const int hc = gl.medium[k];
         const int hb = __ldg(&cp[hc]), he = __ldg(&cp[hc + 1]);
-        bool done = false;
-        for (int e0 = hb; e0 < he && !done; e0 += 32 * GREEDY_U) {  // warp-uniform
-            int r[GREEDY_U], st[GREEDY_U];
-#pragma unroll
-            for (int u = 0; u < GREEDY_U; ++u) {
-                const int e = e0 + u * 32 + lane;
-                r[u] = e < he ? __ldg(&ri[e]) : -1;
-            }
-#pragma unroll
-            for (int u = 0; u < GREEDY_U; ++u) st[u] = r[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
-            while (!done) {  // warp-uniform: the window's free row with the fewest entries
-                int best_s = 0x7fffffff, best_u = -1, best_r = -1;
-#pragma unroll
-                for (int u = 0; u < GREEDY_U; ++u)
-                    if (st[u] >= 0 && (st[u] < best_s || best_u < 0)) { best_s = st[u]; best_u = u; best_r = r[u]; }
-                if (!__any_sync(bmd::FULL, best_u >= 0)) break;  // none left: the next window
-                const int least = __reduce_min_sync(bmd::FULL, best_u >= 0 ? best_s : 0x7fffffff);
-                const int l = __ffs(__ballot_sync(bmd::FULL, best_u >= 0 && best_s == least)) - 1;
-                int won = 0;
-                if (lane == l) {
-                    won = atomicCAS(&state[best_r], best_s, GREEDY_TAKEN) == best_s;
-                    if (won) {
-                        rm[best_r] = hc;
-                        cm[hc] = best_r;
-                    }
-#pragma unroll
-                    for (int u = 0; u < GREEDY_U; ++u)
-                        if (u == best_u) st[u] = GREEDY_TAKEN;
-                }
-                done = __shfl_sync(bmd::FULL, won, l) != 0;
-            }
+        const int r = bmd::greedy_warp(
+            ri + hb, he - hb, [&](int k) { return bmd::ld_volatile(&state[k]); },
+            [&](int k, int seen) { return atomicCAS(&state[k], seen, GREEDY_TAKEN) == seen; });
+        if (r >= 0 && lane == 0) {
+            rm[r] = hc;
+            cm[hc] = r;
         }
     }
 }
@@ -766,6 +705,8 @@ struct bm_ctx {
     int coop_grid[4] = {0, 0, 0, 0};  // blocks of k_match<false, true>, <true, true>, <true, true, true>;
                                       // k_greedy_rounds
     int block = kDefaultBlock;
+    bool solo_ready = false;     // the one-block and one-cluster kernels are set up (configure_solo)
+    bool solo_clusters = false;  // the device holds a cluster of kSoloBlocks
     // deterministic option: allocated on its first use, [dkey nc][ekey nr][ecand nr]
     void* det_arena = nullptr;
     unsigned long long* dkey = nullptr;
@@ -810,6 +751,69 @@ int grid_for(bm_ctx* ctx, int n) {  // plain launches: enough blocks to fill the
     return (int)(want < cap ? want : cap);
 }
 
+// Small graphs run on one block or one cluster of 16 blocks (bm_solo.cuh): the default mode with the
+// launch geometry and the barrier limit left to the library.  Returns the blocks, 0 for other graphs.
+// Cheap matching + search, us, on the grid / one block / 16 blocks (one GB300): 100 rows 137 / 66 / -;
+// 1,000 rows (2.8 k entries) 166 / 92 / 95; 3,000 rows (9 k) 240 / 133 / 127; 10,000 rows (45 k)
+// 374 / 372 / 223; 20,000 rows 344 / - / 208; 60,000 rows 463 / - / 391, but 551 / - / 662 for its search
+// from the empty matching, whose levels are wide.
+constexpr int kSoloBlocks = 16;
+constexpr int64_t kSoloOneBlock = 4096;    // entries up to which one block is faster than 16
+constexpr int32_t kSoloMaxSide = 32768;    // rows and columns up to which 16 blocks are faster than the grid
+constexpr int64_t kSoloMaxEdges = 393216;  // ... and entries (8 MB of L2-resident rows is the grid's)
+
+int solo_cluster(const bm_ctx* ctx) {
+    if (ctx->nr > kSoloMaxSide || ctx->nc > kSoloMaxSide || ctx->nnz > kSoloMaxEdges || ctx->opt.block_size != 0 ||
+        ctx->opt.blocks_per_sm != 0 || ctx->opt.deterministic)
+        return 0;
+    const int C = ctx->nnz > kSoloOneBlock && ctx->nc >= 32 * kSoloBlocks ? kSoloBlocks : 1;
+    if (C > 1 && !ctx->solo_clusters) return 0;
+    if (bms1::Layout(ctx->nr, ctx->nc, ctx->nnz, C).bytes > (unsigned)bms1::SOLO_SMEM) return 0;
+    return C;
+}
+
+void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int C, size_t smem, cudaStream_t st) {
+    cfg.gridDim = dim3((unsigned)C);
+    cfg.blockDim = dim3(bms1::SOLO_T);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+}
+
+// Launches a kernel as one cluster of C blocks.
+template <class... A>
+cudaError_t launch_cluster(void (*kernel)(A...), int C, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    cluster_config(cfg, at, C, smem, st);
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// Once per context: the kernels' shared memory limit, and whether the device can hold their cluster.
+int32_t configure_solo(bm_ctx* ctx) {
+    if (ctx->solo_ready) return BM_OK;
+    auto prepare = [&](auto kernel) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bms1::SOLO_SMEM);
+        return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    };
+    BM_CUDA(ctx, prepare(bms1::k_solo<1>));
+    BM_CUDA(ctx, prepare(bms1::k_solo<kSoloBlocks>));
+    BM_CUDA(ctx, prepare(bms1::k_solo_greedy<1>));
+    BM_CUDA(ctx, prepare(bms1::k_solo_greedy<kSoloBlocks>));
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    cluster_config(cfg, at, kSoloBlocks, bms1::SOLO_SMEM, ctx->stream);
+    int n = 0;
+    ctx->solo_clusters = cudaOccupancyMaxActiveClusters(&n, bms1::k_solo<kSoloBlocks>, &cfg) == cudaSuccess && n > 0;
+    (void)cudaGetLastError();
+    ctx->solo_ready = true;
+    return BM_OK;
+}
+
 int32_t configure(bm_ctx* ctx) {
     ctx->block = ctx->opt.block_size ? ctx->opt.block_size : kDefaultBlock;
     for (int wr = 0; wr < 4; ++wr) {
@@ -827,7 +831,7 @@ int32_t configure(bm_ctx* ctx) {
         if (per_sm < 1 || per_sm * ctx->num_sms > 2047) return BM_ERR_UNSUPPORTED;
         ctx->coop_grid[wr] = per_sm * ctx->num_sms;
     }
-    return BM_OK;
+    return configure_solo(ctx);
 }
 
 Params make_params(bm_ctx* ctx, bool bfs_only) {
@@ -1043,9 +1047,8 @@ int32_t run(bm_ctx* ctx, bool bfs_only) {
     return BM_OK;
 }
 
-int32_t finish(bm_ctx* ctx, int32_t* card_out, bm_stats* stats) {
-    int32_t rc = sync_ctl(ctx);
-    if (rc) return rc;
+// Outcome of the launch whose control block is in ctx->h_ctl; solo: it was k_solo's.
+int32_t report(bm_ctx* ctx, bool solo, int32_t* card_out, bm_stats* stats) {
     const Ctl& h = *ctx->h_ctl;
     const int32_t status = h.status != 0 ? h.status : h.err;
     if (status < 0) ctx->sticky = status;
@@ -1067,12 +1070,46 @@ int32_t finish(bm_ctx* ctx, int32_t* card_out, bm_stats* stats) {
         stats->alternate_steps = h.alt_steps;
         stats->kernel_ns = h.kernel_ns;
         stats->roots = h.roots;
-        if (ctx->opt.driver == BM_DRIVER_PERSISTENT) {
+        if (solo) {
+            stats->grid = solo_cluster(ctx);
+            stats->block = bms1::SOLO_T;
+        } else if (ctx->opt.driver == BM_DRIVER_PERSISTENT) {
             stats->grid = ctx->coop_grid[ctx->opt.deterministic ? 2 : ctx->opt.bfs == BM_GPUBFS_WR ? 1 : 0];
             stats->block = ctx->block;
         }
     }
     return status;
+}
+
+int32_t finish(bm_ctx* ctx, int32_t* card_out, bm_stats* stats) {
+    int32_t rc = sync_ctl(ctx);
+    if (rc) return rc;
+    return report(ctx, false, card_out, stats);
+}
+
+bool solo_match(const bm_ctx* ctx) {
+    return solo_cluster(ctx) > 0 && ctx->opt.mode == BM_APFB && ctx->opt.bfs == BM_GPUBFS_WR &&
+           ctx->opt.driver == BM_DRIVER_PERSISTENT && ctx->opt.wr_one_endpoint == 1 && ctx->opt.wait_timeout_ns == 0;
+}
+
+// The whole search on one block from (rm_src, cm_src); the outcome is in
+// ctx->h_ctl when the stream has been waited for.
+int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool check_src, bool check_err,
+                 int32_t* rm_out, int32_t* cm_out, int32_t* card_out, bm_stats* stats) {
+    const Params p = make_params(ctx, false);
+    const bms1::SoloArgs a{rm_src, cm_src, rm_out, cm_out, ctx->h_ctl, check_src ? 1 : 0, check_err ? 1 : 0};
+    const int C = solo_cluster(ctx);
+    const size_t smem = bms1::Layout(ctx->nr, ctx->nc, ctx->nnz, C).bytes;
+    BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo<1> : bms1::k_solo<kSoloBlocks>, C, smem, ctx->stream, p, a,
+                                (long long)ctx->nnz));
+    BM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return report(ctx, true, card_out, stats);
+}
+
+// The context's matching := empty (rmatch and cmatch lie next to each other).
+int32_t clear_matching(bm_ctx* ctx) {
+    BM_CUDA(ctx, cudaMemsetAsync(ctx->rmatch, 0xff, (size_t)((char*)(ctx->cmatch + ctx->nc) - (char*)ctx->rmatch), ctx->stream));
+    return BM_OK;
 }
 
 }  // namespace
@@ -1255,6 +1292,14 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
     if (!ctx) return BM_ERR_INVALID_ARG;
     if (ctx->sticky || !ctx->csr_ready) return BM_ERR_STATE;
     cudaStream_t st = ctx->stream;
+    if (const int C = solo_cluster(ctx)) {
+        const size_t smem = 128 * ((((size_t)ctx->nr + 31) / 32 + C - 1) / C);
+        BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo_greedy<1> : bms1::k_solo_greedy<kSoloBlocks>, C, smem, st,
+                                    make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl));
+        BM_CUDA(ctx, cudaStreamSynchronize(st));
+        if (card_out) *card_out = ctx->h_ctl->card;
+        return BM_OK;
+    }
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     if (ctx->nc && ctx->opt.deterministic) {
         // proposal rounds: the same matching on every run and launch geometry
@@ -1289,11 +1334,7 @@ int32_t bm_set_matching(bm_ctx* ctx, const int32_t* rmatch, const int32_t* cmatc
     if (!ctx || ((rmatch == nullptr) != (cmatch == nullptr))) return BM_ERR_INVALID_ARG;
     if (ctx->sticky) return BM_ERR_STATE;
     cudaStream_t st = ctx->stream;
-    if (!rmatch) {
-        BM_CUDA(ctx, cudaMemsetAsync(ctx->rmatch, 0xff, 4 * (size_t)ctx->nr, st));
-        BM_CUDA(ctx, cudaMemsetAsync(ctx->cmatch, 0xff, 4 * (size_t)ctx->nc, st));
-        return BM_OK;
-    }
+    if (!rmatch) return clear_matching(ctx);
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     if (ctx->nr) BM_CUDA(ctx, cudaMemcpyAsync(ctx->rmatch, rmatch, 4 * (size_t)ctx->nr, cudaMemcpyDeviceToDevice, st));
     if (ctx->nc) BM_CUDA(ctx, cudaMemcpyAsync(ctx->cmatch, cmatch, 4 * (size_t)ctx->nc, cudaMemcpyDeviceToDevice, st));
@@ -1325,6 +1366,8 @@ int32_t bm_match(bm_ctx* ctx, int32_t* rmatch_out, int32_t* cmatch_out, int32_t*
     bmi::NvtxRange nvtx_range("bm_match");
     if (!ctx) return BM_ERR_INVALID_ARG;
     if (ctx->sticky || !ctx->csr_ready) return BM_ERR_STATE;
+    if (solo_match(ctx))
+        return run_solo(ctx, ctx->rmatch, ctx->cmatch, false, false, rmatch_out, cmatch_out, card_out, stats);
     cudaStream_t st = ctx->stream;
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     int32_t rc = run(ctx, false);
@@ -1339,6 +1382,15 @@ int32_t bm_match_from(bm_ctx* ctx, const int32_t* rmatch0, const int32_t* cmatch
     bmi::NvtxRange nvtx_range("bm_match_from");
     if (!ctx || !rmatch0 || !cmatch0) return BM_ERR_INVALID_ARG;
     if (ctx->sticky || !ctx->csr_ready) return BM_ERR_STATE;
+    if (solo_match(ctx)) {
+        const int32_t rc1 = run_solo(ctx, rmatch0, cmatch0, true, false, rmatch_out, cmatch_out, card_out, stats);
+        if (rc1 != BM_ERR_INVALID_MATCHING) return rc1;
+        ctx->sticky = 0;  // bad input is not a broken context: leave the empty matching installed
+        const int32_t rc2 = clear_matching(ctx);
+        if (rc2) return rc2;
+        cudaStreamSynchronize(ctx->stream);
+        return rc1;
+    }
     cudaStream_t st = ctx->stream;
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     // copy and check in one launch; the check reports through the control block, and the
@@ -1390,13 +1442,20 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
         if (rc) return rc;
         if (ctx->h_ctl->err) { ctx->csr_ready = false; return ctx->h_ctl->err; }
     }
-    rc = run(ctx, false);
-    if (rc < 0) return rc;
+    const bool solo = solo_match(ctx);
+    if (solo) {
+        rc = run_solo(ctx, ctx->rmatch, ctx->cmatch, false, true, nullptr, nullptr, card_out, stats);
+        if (rc < 0 && rc != BM_ERR_INVALID_CSR && rc != BM_ERR_INVALID_MATCHING) return rc;
+    } else {
+        rc = run(ctx, false);
+        if (rc < 0) return rc;
+    }
     if (h_rmatch) {
         if (ctx->nr) BM_CUDA(ctx, cudaMemcpyAsync(h_rmatch, ctx->rmatch, 4 * (size_t)ctx->nr, cudaMemcpyDeviceToHost, st));
         if (ctx->nc) BM_CUDA(ctx, cudaMemcpyAsync(h_cmatch, ctx->cmatch, 4 * (size_t)ctx->nc, cudaMemcpyDeviceToHost, st));
     }
-    rc = finish(ctx, card_out, stats);
+    if (!solo) rc = finish(ctx, card_out, stats);
+    else if (h_rmatch) BM_CUDA(ctx, cudaStreamSynchronize(st));
     if (rc == BM_ERR_INVALID_CSR || rc == BM_ERR_INVALID_MATCHING) {
         ctx->csr_ready = false;
         ctx->sticky = 0;  // bad input is not a broken context
