@@ -56,6 +56,7 @@ struct BatchParams {
     int32_t* pred;
     int2* queue;
     int32_t* endpoints;
+    const uint8_t* rdeg8;      // per row: its number of entries, at most 255
     unsigned long long* dkey;  // deterministic option: per column, per row; rows listed per level
     unsigned long long* ekey;
     int32_t* ecand;
@@ -92,6 +93,7 @@ __global__ void __launch_bounds__(1024, 1) k_batch(BatchParams bp) {
         p.pred = bp.pred + ro;
         p.queue = bp.queue + co;
         p.endpoints = bp.endpoints + ro;
+        p.rdeg8 = bp.rdeg8 + ro;
         p.mode = bp.mode;
         p.one_ep = bp.one_ep;
         p.chk = &bp.ctl->err;
@@ -152,10 +154,11 @@ __global__ void __launch_bounds__(1024, 1) k_batch(BatchParams bp) {
     }
 }
 
-// Validates every graph's local CSR (one block per graph at a time).
+// Validates every graph's local CSR (one block per graph at a time) and counts the rows' entries
+// in rdeg (all rows of the batch, zero before).
 __global__ void k_batch_check(int G, const int32_t* n_rows, const int32_t* n_cols, const int64_t* row_off,
                               const int64_t* col_off, const int64_t* edge_off, const int32_t* col_ptr,
-                              const int32_t* row_idx, BatchCtl* ctl) {
+                              const int32_t* row_idx, int32_t* rdeg, BatchCtl* ctl) {
     for (int g = blockIdx.x; g < G; g += gridDim.x) {
         const int nr = n_rows[g], nc = n_cols[g];
         const int32_t* cp = col_ptr + col_off[g] + g;
@@ -169,11 +172,20 @@ __global__ void k_batch_check(int G, const int32_t* n_rows, const int32_t* n_col
         if (nc >= 0 && col_off[g + 1] - col_off[g] == nc) {
             for (int c = threadIdx.x; c < nc; c += blockDim.x)
                 if (cp[c + 1] < cp[c]) bad = true;
-            for (long long e = threadIdx.x; e < nnz; e += blockDim.x)
-                if (ri[e] < 0 || ri[e] >= nr) bad = true;
+            const bool rows_ok = nr >= 0 && row_off[g + 1] - row_off[g] == nr;
+            for (long long e = threadIdx.x; e < nnz; e += blockDim.x) {
+                const int r = ri[e];
+                if (r < 0 || r >= nr) bad = true;
+                else if (rows_ok) atomicAdd(&rdeg[row_off[g] + r], 1);
+            }
         }
         if (bad) atomicCAS(&ctl->err, 0, BM_ERR_INVALID_CSR);
     }
+}
+
+__global__ void k_batch_rdeg8(long long n, const int32_t* rdeg, uint8_t* rdeg8) {
+    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n; r += (long long)gridDim.x * blockDim.x)
+        rdeg8[r] = (uint8_t)min(rdeg[r], 255);
 }
 
 }  // namespace
@@ -188,6 +200,7 @@ struct bm_batch {
     int32_t *order = nullptr, *level = nullptr, *root = nullptr, *pred = nullptr, *endpoints = nullptr,
             *card = nullptr, *status = nullptr, *phases = nullptr;
     int2* queue = nullptr;
+    uint8_t* rdeg8 = nullptr;
     BatchCtl* ctl = nullptr;
     BatchCtl* h_ctl = nullptr;
     cudaGraph_t graph = nullptr;
@@ -235,6 +248,7 @@ BatchParams batch_params(bm_batch* b, int32_t* rmatch, int32_t* cmatch, int gree
     bp.pred = b->pred;
     bp.queue = b->queue;
     bp.endpoints = b->endpoints;
+    bp.rdeg8 = b->rdeg8;
     if (b->det_arena) {
         const size_t cols = (size_t)(b->total_cols ? b->total_cols : 1), rows = (size_t)(b->total_rows ? b->total_rows : 1);
         char* a = (char*)b->det_arena;
@@ -361,6 +375,7 @@ int32_t bm_batch_create(const bm_batch_desc* desc, void* stream, const bm_option
     const size_t o_q = off; off += al(8 * C);
     const size_t o_pd = off; off += al(4 * R);
     const size_t o_ep = off; off += al(4 * R);
+    const size_t o_rd = off; off += al(R);
     const size_t det_bytes = al(8 * C) + al(8 * R) + 4 * R;
     if (cudaMalloc(&b->arena, off) != cudaSuccess || cudaMallocHost((void**)&b->h_ctl, sizeof(BatchCtl)) != cudaSuccess ||
         (o.deterministic && cudaMalloc(&b->det_arena, det_bytes) != cudaSuccess)) {
@@ -379,6 +394,7 @@ int32_t bm_batch_create(const bm_batch_desc* desc, void* stream, const bm_option
     b->queue = (int2*)(a + o_q);
     b->pred = (int32_t*)(a + o_pd);
     b->endpoints = (int32_t*)(a + o_ep);
+    b->rdeg8 = (uint8_t*)(a + o_rd);
     int32_t rc = configure_batch(b);
     if (rc) { bm_batch_destroy(b); return rc; }
     if (cudaMemcpyAsync(b->order, order.data(), 4 * (size_t)G, cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -388,8 +404,11 @@ int32_t bm_batch_create(const bm_batch_desc* desc, void* stream, const bm_option
         return BM_ERR_CUDA;
     }
     if (G > 0) {
+        // the rows' entry counts (for the cheap matching) pass through the endpoint lists' space
+        cudaMemsetAsync(b->endpoints, 0, 4 * R, st);
         k_batch_check<<<b->num_sms * 4, 256, 0, st>>>(G, desc->n_rows, desc->n_cols, desc->row_off, desc->col_off, desc->edge_off,
-                                                     desc->col_ptr, desc->row_idx, b->ctl);
+                                                     desc->col_ptr, desc->row_idx, b->endpoints, b->ctl);
+        k_batch_rdeg8<<<b->num_sms * 4, 256, 0, st>>>((long long)b->total_rows, b->endpoints, b->rdeg8);
     }
     if (cudaGetLastError() != cudaSuccess ||
         cudaMemcpyAsync(b->h_ctl, b->ctl, sizeof(BatchCtl), cudaMemcpyDeviceToHost, st) != cudaSuccess ||

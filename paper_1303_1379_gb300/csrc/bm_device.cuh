@@ -155,6 +155,7 @@ struct Params {
     // the level array's tests and claims
     unsigned* vis;
     unsigned* srv;
+    const uint8_t* rdeg8;  // ... and per row its number of entries, at most 255 (nullable)
 };
 
 // Per-block shared state of the steps.
@@ -1488,6 +1489,80 @@ __device__ __forceinline__ void step_release_endpoints(const Params& p, int n_ep
 }
 
 // ------------------------------------------------------------------ one graph, one block
+// The cheap matching of one graph by one block with the rows' marks in shared
+// memory (p.vis: one bit per matched row, at most SB_MAX_COLS rows): the
+// whole-GPU passes' choice (the least-listed free row of a rotated list, columns
+// scattered), but a column looks at GW rows of its list at a time and takes the
+// first window's, and all degrees go in one pass.  A thread takes two columns at
+// a time, their loads in flight together.  (4,096 graphs, ms for the launch: first
+// free row 5.53, this 4.86, shortest lists first in three passes 5.33, four rows a
+// window 5.31, columns in order 4.76 -- but 64 meshes of 150 x 150 and more take
+// 16.4 / 3.6 / - / 3.4 / 7.0.)
+template <bool NC>
+__device__ __forceinline__ void block_greedy_sb(const Params& p) {
+    constexpr int GW = 8, GU = 2;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, nc = p.nc;
+    const unsigned tiles = ((unsigned)nc + 31) >> 5;
+    const int bits = tiles > 1 ? 32 - __clz(tiles - 1) : 0;  // 2^bits >= tiles
+    for (unsigned k0 = warp; k0 < (1u << bits); k0 += GU * nwarps) {
+        int c[GU], beg[GU], deg[GU], m0[GU], pos[GU], rot[GU];
+#pragma unroll
+        for (int v = 0; v < GU; ++v) {
+            const unsigned k = k0 + v * nwarps;
+            const unsigned tile = k < (1u << bits) ? scatter_bits(k, bits) : tiles;
+            c[v] = tile < tiles ? scatter_lane(tile, lane) : nc;
+            m0[v] = 0;
+            beg[v] = deg[v] = pos[v] = 0;
+            if (c[v] < nc) {
+                m0[v] = __ldcg(&p.cmatch[c[v]]);
+                beg[v] = ld_csr<NC>(&p.col_ptr[c[v]]);
+                deg[v] = ld_csr<NC>(&p.col_ptr[c[v] + 1]) - beg[v];
+            }
+            rot[v] = (int)__umulhi(hash32((unsigned)c[v]), (unsigned)deg[v]);
+        }
+#pragma unroll
+        for (int v = 0; v < GU; ++v)
+            if (m0[v] != -1) deg[v] = 0;
+        for (;;) {
+            int r[GU][GW], d[GU][GW];
+#pragma unroll
+            for (int v = 0; v < GU; ++v)
+#pragma unroll
+                for (int u = 0; u < GW; ++u) {
+                    const int j = pos[v] + u + rot[v];
+                    r[v][u] = pos[v] + u < deg[v] ? ld_csr<NC>(&p.row_idx[beg[v] + (j < deg[v] ? j : j - deg[v])]) : -1;
+                }
+#pragma unroll
+            for (int v = 0; v < GU; ++v)
+#pragma unroll
+                for (int u = 0; u < GW; ++u) d[v][u] = r[v][u] >= 0 && !sb_test(p.vis, r[v][u]) ? p.rdeg8[r[v][u]] : 256;
+            bool more = false;
+#pragma unroll
+            for (int v = 0; v < GU; ++v) {
+                for (;;) {  // the window's free row with the fewest entries that no one takes meanwhile
+                    int best = 256, row = -1;
+#pragma unroll
+                    for (int u = 0; u < GW; ++u)
+                        if (d[v][u] < best) { best = d[v][u]; row = r[v][u]; }
+                    if (row < 0) break;
+                    if (sb_claim(p.vis, row)) {
+                        p.rmatch[row] = c[v];
+                        p.cmatch[c[v]] = row;
+                        deg[v] = 0;
+                        break;
+                    }
+#pragma unroll
+                    for (int u = 0; u < GW; ++u)
+                        if (r[v][u] == row) d[v][u] = 256;
+                }
+                pos[v] += GW;
+                more |= pos[v] < deg[v];
+            }
+            if (!more) break;
+        }
+    }
+}
+
 // InitBfsArray over all columns of one graph by one block (4 columns per
 // thread in flight): column half of FixMatching, level / root init, unmatched
 // columns with rows appended to the queue as roots.  Returns the roots in
@@ -1605,7 +1680,9 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
     // (not the sum of its walks).  A column's row range is loaded beside its match.
     // rows_sb: a row's test and claim are a bitmap read and atomicOr in shared
     // memory, and the winner stores both matches (read only after the block barrier).
-    if (greedy) {
+    if (greedy && rows_sb && p.rdeg8) {
+        block_greedy_sb<NC>(p);
+    } else if (greedy) {
         constexpr int GW = 8, GU = 2;
         for (int base = 0; base < nc; base += GU * T) {
             int c[GU], pos[GU], e[GU];

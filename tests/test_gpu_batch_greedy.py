@@ -1,0 +1,54 @@
+"""The block routine's cheap matching (entry counts saturating at 255, lists on
+both sides of its 8-row window, rows beyond the shared-memory marks, partial
+starts) and the batch's default geometry on both sides of its limit."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1303_1379_gb300 import bmatch, synth
+
+from helpers import csr_from_edges
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def to_batch(graphs):
+    off = [np.concatenate([[0], np.cumsum([f(g) for g in graphs])]).astype(np.int64)
+           for f in (lambda g: g.n_rows, lambda g: g.n_cols, lambda g: g.nnz)]
+    return synth.Batch(np.array([g.n_rows for g in graphs], np.int32), np.array([g.n_cols for g in graphs], np.int32),
+                       *off, np.concatenate([g.col_ptr for g in graphs]), np.concatenate([g.row_idx for g in graphs]))
+
+
+def graphs_at_the_edges():
+    rng = np.random.default_rng(9)
+    out = [csr_from_edges(1, 1, [(0, 0)]), csr_from_edges(3, 40, [])]
+    # every column lists rows 0-6 and one of the others: rows of more than 255 entries, lists of 1, 8 and 9
+    out.append(csr_from_edges(400, 390, [(r, c) for c in range(390) for r in (*range(7), 7 + c)]))
+    out.append(csr_from_edges(500, 300, [(int(r), c) for c in range(300) for r in rng.choice(500, (1, 7, 8, 9, 16, 17)[c % 6], replace=False)]))
+    out.append(synth.uniform_graph(61440, 9000, 3, seed=1))  # the last row count with marks in shared memory
+    out.append(synth.uniform_graph(61441, 9000, 3, seed=1))
+    out.append(synth.stencil_graph(60, 360, 0.2, seed=2))
+    return out
+
+
+@pytest.mark.parametrize("partial", [False, True])
+def test_batch_cheap_matching_at_its_edges(partial):
+    graphs = graphs_at_the_edges()
+    b = to_batch(graphs)
+    want = [oracle.hopcroft_karp(g.n_rows, g.n_cols, g.col_ptr, g.row_idx)[2] for g in graphs]
+    rm0, cm0 = np.full(int(b.row_off[-1]), -1, np.int32), np.full(int(b.col_off[-1]), -1, np.int32)
+    if partial:
+        for k, g in enumerate(graphs):
+            _, cg, _ = oracle.greedy(g.n_rows, g.n_cols, g.col_ptr, g.row_idx)
+            for c in np.flatnonzero(cg >= 0)[::3]:
+                rm0[b.row_off[k] + cg[c]], cm0[b.col_off[k] + c] = c, cg[c]
+    with bmatch.Batch.from_synth(b) as bb:
+        rm, cm = torch.from_numpy(rm0).cuda(), torch.from_numpy(cm0).cuda()
+        card = torch.empty(len(graphs), dtype=torch.int32, device="cuda")
+        bb.match(rm, cm, greedy=True, card_out=card)
+    assert card.cpu().tolist() == want
+    rm, cm = rm.cpu().numpy(), cm.cpu().numpy()
+    for k, g in enumerate(graphs):
+        assert oracle.validate(g.n_rows, g.n_cols, g.col_ptr, g.row_idx, rm[b.row_off[k]:b.row_off[k + 1]],
+                               cm[b.col_off[k]:b.col_off[k + 1]]) == (0, want[k])
