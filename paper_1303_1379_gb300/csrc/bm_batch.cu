@@ -192,7 +192,7 @@ __global__ void k_batch_rdeg8(long long n, const int32_t* rdeg, uint8_t* rdeg8) 
 
 struct bm_batch {
     bm_batch_desc d{};
-    int64_t total_rows = 0, total_cols = 0, total_edges = 0;
+    int64_t total_rows = 0, total_cols = 0, total_edges = 0, max_edges = 0;
     cudaStream_t stream = nullptr;
     bm_options opt{};
     int block = 512, grid = 0, num_sms = 0;
@@ -264,7 +264,13 @@ BatchParams batch_params(bm_batch* b, int32_t* rmatch, int32_t* cmatch, int gree
 }
 
 int32_t configure_batch(bm_batch* b) {
-    b->block = b->opt.block_size ? b->opt.block_size : 512;
+    // Without a size from the caller: two blocks of 512 threads an SM while the whole batch is what takes
+    // the time, one of 1,024 when the largest graphs are (they run first, on a block each, and the launch
+    // lasts as long as they do): one GB300, graphs of 100 to 50,000 rows, ms at 512 / 1,024 threads: 512
+    // graphs 2.46 / 1.59, 1,024 2.9 / 2.2, 2,048 3.5 / 3.1, 4,096 4.86 / 5.00; 48 from the empty matching
+    // 2.35 / 1.41.  4,096 such graphs hold 2.3 times num_sms x the largest one's entries, 2,048 half that.
+    const bool few = b->total_edges < 2 * (int64_t)b->num_sms * b->max_edges;
+    b->block = b->opt.block_size ? b->opt.block_size : few && b->opt.blocks_per_sm == 0 ? 1024 : 512;
     int per_sm = 0;
     cudaError_t e = b->opt.deterministic
                         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch<true, true>, b->block, 0)
@@ -356,6 +362,7 @@ int32_t bm_batch_create(const bm_batch_desc* desc, void* stream, const bm_option
     b->total_rows = ro[G];
     b->total_cols = co[G];
     b->total_edges = eo[G];
+    for (int g = 0; g < G; ++g) b->max_edges = std::max(b->max_edges, eo[g + 1] - eo[g]);
     std::vector<int32_t> order(G);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {

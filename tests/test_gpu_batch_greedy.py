@@ -52,3 +52,18 @@ def test_batch_cheap_matching_at_its_edges(partial):
     for k, g in enumerate(graphs):
         assert oracle.validate(g.n_rows, g.n_cols, g.col_ptr, g.row_idx, rm[b.row_off[k]:b.row_off[k + 1]],
                                cm[b.col_off[k]:b.col_off[k + 1]]) == (0, want[k])
+
+
+@pytest.mark.parametrize("n,block", [(40, 1024), (700, 512)])
+def test_batch_default_geometry(n, block):
+    graphs = [synth.uniform_graph(200, 210, 4, seed=k) for k in range(n)]
+    b = to_batch(graphs)
+    with bmatch.Batch.from_synth(b) as bb:
+        rm = torch.full((int(b.row_off[-1]),), -1, dtype=torch.int32, device="cuda")
+        cm = torch.full((int(b.col_off[-1]),), -1, dtype=torch.int32, device="cuda")
+        card = torch.empty(n, dtype=torch.int32, device="cuda")
+        _, st = bb.match(rm, cm, card_out=card)
+    assert st["block"] == block
+    for k in (0, n - 1):
+        g = graphs[k]
+        assert int(card[k]) == oracle.hopcroft_karp(g.n_rows, g.n_cols, g.col_ptr, g.row_idx)[2]
