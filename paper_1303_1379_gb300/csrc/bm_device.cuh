@@ -78,6 +78,9 @@ constexpr int CARRY_PHASES = 20;
 constexpr int CUT_PHASES = 10;
 constexpr int CUT_MIN = 5, CUT_MAX = 24;  // levels of a phase after which it may be cut
 constexpr int CUT_RATIO = 16;             // ... if the next has at most 1 / CUT_RATIO of the forest's columns
+constexpr int CUT_FOUND = 32;             // ... and blocks of the grid have found endpoints this often (the next
+                                          // phase's start is not worth a few; 16 to 48 alike, R-MAT scale 21
+                                          // 645 -> 630 us, 2000 x 2000 mesh 56 -> 50 ms against 1)
 
 // Control block in device memory, cleared before every launch.  Per-step
 // counters rotate over three slots: step s appends to slot s % 3 and clears
@@ -594,12 +597,15 @@ __device__ __forceinline__ void step_next_roots(const Params& p, const int2* q, 
 // the other trees go back to "unvisited", and so do the rows they were reached
 // through (rv_free: a stamp below the phases').  A root is served when its
 // level slot is not L0: -(row), or L0 - 1 once its own entry was reset here.
-// Runs beside Alternate's walks, like step_next_roots.
-__device__ __forceinline__ void step_carry(const Params& p, const int2* q, int tail, int2* q_next, int slot,
+// Runs beside Alternate's walks, like step_next_roots: the n_ep walks are the first
+// blocks', so the entries are dealt from the first block without one on.
+__device__ __forceinline__ void step_carry(const Params& p, const int2* q, int tail, int2* q_next, int n_ep, int slot,
                                            bool keep_trees, int rv_free, Smem& sm) {
     const int T = blockDim.x;
     const int per = T <= QBUF / 4 ? 4 : QBUF / T;  // entries per thread per pass: at most QBUF a block
-    for (int base = blockIdx.x * per * T; base < tail; base += gridDim.x * per * T) {  // block-uniform
+    const int walkers = min((n_ep + T - 1) / T, (int)gridDim.x);
+    const int me = (int)(blockIdx.x + gridDim.x - walkers) % (int)gridDim.x;
+    for (int base = me * per * T; base < tail; base += gridDim.x * per * T) {  // block-uniform
         int2 e[4];
         int lv[4];
 #pragma unroll

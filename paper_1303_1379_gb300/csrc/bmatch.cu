@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
 
         // ---- BFS, level by level (Algorithm 1 inner loop)
         int qb = 0, qe = n_front, lvl = L0, tail = n_front;
-        bool any_ep = false;
+        int ep_blocks = 0;  // blocks that found endpoints, added up over the phase's levels
         if (leader) { ls.levels = 0; ls.first_ep = 0; ls.last_ep = 0; ls.roots_total += n_roots; }
         for (;;) {
             const int s2 = step++;
@@ -143,9 +143,9 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
             tail = qe + nq;
             if (nq == 0) break;              // no vertex inserted
             if (p.mode == 1 && found) break;  // APsB: stop at the first level with a path
-            any_ep |= found;
+            ep_blocks += sm.bc_b;
             // what is left of a carried search is narrow: augment, and search on from its trees
-            if (graft && any_ep && phases <= bmd::CUT_PHASES && lvl - L0 + 1 >= CUT_MIN && lvl - L0 + 1 <= CUT_MAX &&
+            if (graft && ep_blocks >= CUT_FOUND && phases <= bmd::CUT_PHASES && lvl - L0 + 1 >= CUT_MIN && lvl - L0 + 1 <= CUT_MAX &&
                 (long long)nq * CUT_RATIO <= tail)
                 break;
             qb = qe;
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
             }
             step_alternate_disjoint(p, n_ep, tail + 2, DET ? -1 : p.stamp_base);
             if (phases >= CARRY_PHASES) carry = false;
-            if (graft) step_carry(p, qcur, tail, qnext, s3 % 3, carry, p.stamp_base, sm);
+            if (graft) step_carry(p, qcur, tail, qnext, n_ep, s3 % 3, carry, p.stamp_base, sm);
             else step_next_roots<WR, DET, true>(p, qcur, n_roots, tail, qnext, s3 % 3, sm);
         } else {
             step_alternate(p, n_ep, tail + 2, cnt);
