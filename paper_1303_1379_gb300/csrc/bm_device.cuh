@@ -145,6 +145,7 @@ struct Params {
     int32_t* profile;    // per phase: levels, endpoints, first and last level with an endpoint (nullable)
     long long wait_ns;   // limit of one barrier wait
     long long total_ns;  // limit of the whole launch
+    int32_t pre;         // the first phase was run as a cheap matching, from the empty matching (k_match)
     int32_t stamp_base;  // rvis stamp of phase k is stamp_base + k (k >= 1); above every stamp in rvis
     int32_t* chk;        // range-checked build: error word set when an index is out of range (nullable)
     // deterministic option (nullable otherwise): per column the tree-entry key
@@ -1658,6 +1659,7 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
     // rows that are matched, so the cheap matching tests and claims a row in
     // shared memory instead of loading and CASing its match
     const bool rows_sb = SB && nr <= SB_MAX_COLS;
+    bool matched = false;  // rows_sb: some row of this thread's is
     if (t == 0) sm.ok = 0;
     // ---- rows whose column does not point back are unmatched (row half of FixMatching)
     if (rows_sb) {  // a warp takes 32 consecutive rows and writes their bitmap word
@@ -1671,6 +1673,7 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
             }
             const unsigned w = __ballot_sync(FULL, m != -1);
             if (lane == 0) p.vis[r0 >> 5] = w;
+            matched |= w != 0u;
         }
     } else {
         for (int r = t; r < nr; r += T) {
@@ -1678,7 +1681,11 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
             if (m != -1 && (m < 0 || m >= nc || __ldcg(&p.cmatch[m]) != r)) __stcg(&p.rmatch[r], -1);
         }
     }
-    __syncthreads();
+    // From the empty matching the first level of the first phase gives every column that it can a free row: the
+    // cheap matching, only without its choices, so the cheap matching runs it and the phase ends there (48
+    // graphs of 100 to 50,000 rows from the empty matching: 1.43 -> 0.95 ms).
+    const bool empty = __syncthreads_or(matched) == 0;
+    const bool pre = rows_sb && p.rdeg8 && !greedy && p.mode == 0 && empty;
     // ---- cheap matching (Section 4): unmatched columns claim their first free row.
     // A thread walks the lists of GU columns together, GW rows of each per step,
     // so that GU x GW row loads (and, without rows_sb, then GU x GW match loads)
@@ -1686,7 +1693,7 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
     // (not the sum of its walks).  A column's row range is loaded beside its match.
     // rows_sb: a row's test and claim are a bitmap read and atomicOr in shared
     // memory, and the winner stores both matches (read only after the block barrier).
-    if (greedy && rows_sb && p.rdeg8) {
+    if ((greedy || pre) && rows_sb && p.rdeg8) {
         block_greedy_sb<NC>(p);
     } else if (greedy) {
         constexpr int GW = 8, GU = 2;
@@ -1744,6 +1751,12 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
     int free_total = 0, iso_free = 0;
     block_full_init<WR, NC, SB>(p, sm, cnt, free_total, iso_free);
     int n_roots = sm.qn;
+    if (pre && free_total < nc) {
+        phases = 1;
+        levels_total = 1;
+        eps_total = nc - free_total;
+        if (t == 0) cnt.alt += (unsigned)(nc - free_total);
+    }
     for (;;) {
         card = nc - free_total;
         if (n_roots == 0) break;

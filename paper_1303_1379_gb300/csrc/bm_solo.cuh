@@ -64,6 +64,7 @@ struct SoloArgs {
     Ctl* h_ctl;             // the host's copy of the control block (pinned)
     int32_t check_src;      // check that rm_src / cm_src are in range and inverse to each other
     int32_t check_err;      // p.ctl holds the outcome of input checks queued before
+    int32_t pre;            // the first phase was run as a cheap matching, from the empty matching
 };
 
 // Where a block keeps what, in bytes from its dynamic shared memory's start.
@@ -367,8 +368,22 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
     };
     end_step(true);
     int n_roots = sum_cnt, n_free = sum_eps, n_front = sum_cnt;
-    const int initial = nc - n_free;
+    int initial = nc - n_free;
     int status = flag, phases = 0, no_roots = 0;
+    if (a.pre && initial > 0) {
+        phases = 1;
+        if (leader) {
+            sm.st.levels = sm.st.levels_max = 1;
+            sm.st.eps = initial;
+            sm.st.roots = initial + n_roots;
+            if (p.profile && p.profile_cap > 0) {
+                p.profile[0] = p.profile[2] = p.profile[3] = 1;
+                p.profile[1] = initial;
+            }
+            alt = (unsigned)initial;
+        }
+        initial = 0;
+    }
     bool carry = true;
     int wins = 0;
 

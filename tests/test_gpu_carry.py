@@ -14,7 +14,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 GRAPHS = {
-    "mesh": lambda: synth.stencil_graph(260, 6760, 0.05, seed=11),           # long paths, over 20 phases from nothing
+    "mesh": lambda: synth.stencil_graph(260, 6760, 0.05, seed=11),           # long paths
     "sparse": lambda: synth.uniform_graph(70001, 69997, 4, seed=12),         # many roots that fail
     "rmat": lambda: synth.rmat_graph(16, 1 << 19, seed=13),
     "wide": lambda: synth.uniform_graph(400003, 399989, 5, seed=14),         # levels on both sides of the claim limit
@@ -50,9 +50,15 @@ def test_carried_search_is_maximum(graph, block, per_sm):
 
 
 def test_a_long_search_passes_both_limits():
-    """The mesh from the empty matching takes more phases than are carried."""
-    g = GRAPHS["mesh"]()
+    """A mesh from a one-sided start (every column's first free row) takes more
+    phases than are carried."""
+    g = synth.stencil_graph(500, 25000, 0.05, seed=2)
     cp, ri = to_dev(g)
-    with bmatch.Matcher(g.n_rows, g.n_cols, g.nnz, cp, ri) as m:
-        res = m.match()
-    assert res.card == oracle_max(g) and res.stats["phases"] > 20
+    rm = torch.empty(g.n_rows, dtype=torch.int32, device="cuda")
+    cm = torch.empty(g.n_cols, dtype=torch.int32, device="cuda")
+    with bmatch.Matcher(g.n_rows, g.n_cols, g.nnz, cp, ri, deterministic=1) as m:
+        m.greedy()
+        m.set_options(deterministic=0)
+        res = m.match(rm, cm)
+    assert_maximum(g, rm.cpu().numpy(), cm.cpu().numpy(), res.card, oracle_max(g))
+    assert res.stats["phases"] > 20
