@@ -24,8 +24,9 @@
 //    the level's barrier, so no append waits for a position, and levels are spread
 //    over the blocks by column id.
 // A word's rows that do not fit the block's memory are read from the graph itself.
-// One block of 1,024 threads (C = 1) for the smallest graphs, whose levels are too
-// narrow for more; a cluster spreads the wide levels' instructions and holds larger
+// One block (C = 1) for the smallest graphs, whose levels are too narrow for more, of
+// 512 threads (1,000 rows: 25 us a search, with 1,024 threads 38 us: half as many warps
+// meet at each barrier); a cluster spreads the wide levels' instructions and holds larger
 // graphs.  What a level costs then is a warp's chain of instructions (about 2,500
 // cycles for 64 edges a warp; a narrow level's columns go to all warps), and with
 // C = 16 the barrier with its release (2,000 cycles).
@@ -48,7 +49,8 @@ using bmd::L0;
 using bmd::Params;
 
 typedef unsigned short u16;
-constexpr int SOLO_T = 1024;           // threads of a block
+constexpr int SOLO_T = 1024;           // threads of a cluster's block
+constexpr int SOLO_T1 = 512;           // threads of a single block
 constexpr int SOLO_FREE = 0xffff;      // "unmatched" in 16 bits
 constexpr int SOLO_MAX = 0xfffe;       // rows and columns with a 16-bit id
 constexpr int SOLO_SMEM = 216 * 1024;  // dynamic shared memory of a block
@@ -199,8 +201,8 @@ __device__ __forceinline__ void block_add(unsigned long long* dst, unsigned v) {
     if ((threadIdx.x & 31) == 0 && s) atomicAdd(dst, s);
 }
 
-template <int C>
-__global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long long nnz) {
+template <int C, int T>
+__global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long nnz) {
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ SoloShared sm;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, wb = t & ~31;
@@ -232,9 +234,9 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
         if (a.check_err) sm.flag = p.ctl->err;
         else if (rank == 0) p.ctl->err = 0;
     }
-    for (int w = t; w < words; w += SOLO_T) vis[w] = srv[w] = 0u;
-    for (int w = t; w < 2 * (int)lay.own_cw; w += SOLO_T) fresh[w] = 0u;
-    for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += SOLO_T) rcl[w] = 0u;
+    for (int w = t; w < words; w += T) vis[w] = srv[w] = 0u;
+    for (int w = t; w < 2 * (int)lay.own_cw; w += T) fresh[w] = 0u;
+    for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += T) rcl[w] = 0u;
     cluster_sync<C>();  // every block has started and cleared its shared memory
     const int input_err = sm.flag;
     const bool leader = rank == 0 && t == 0;  // keeps the statistics, in shared memory
@@ -242,7 +244,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
     // ---- the matching and the own columns' rows to shared memory; unmatched columns with rows are the first roots
     if (input_err == 0) {
         bool bad = false;
-        for (int r = t; r < nr; r += SOLO_T) {
+        for (int r = t; r < nr; r += T) {
             int c = __ldg(&a.rm_src[r]);
             if (a.check_src && owner<C>(r) == rank && c != -1 && (c < 0 || c >= nc || __ldg(&a.cm_src[c]) != r)) {
                 bad = true;
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
             rm[r] = (u16)(c < 0 ? SOLO_FREE : c);
         }
         int nf = 0, nroot = 0;
-        for (int ow = warp; ow < (int)lay.own_cw; ow += SOLO_T / 32) {
+        for (int ow = warp; ow < (int)lay.own_cw; ow += T / 32) {
             const int w = ow * C + rank, c = w * 32 + lane, sl = ow * 32 + lane;
             int b = 0, d = 0, r = 0;
             if (c < nc) {
@@ -328,7 +330,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
         }
         // a warp takes four own words at a time, a lane a column of each; a column of more than PART rows is
         // listed once for each part
-        for (int ow0 = 4 * warp; ow0 < (int)lay.own_cw; ow0 += 4 * (SOLO_T / 32)) {  // warp-uniform
+        for (int ow0 = 4 * warp; ow0 < (int)lay.own_cw; ow0 += 4 * (T / 32)) {  // warp-uniform
             unsigned f[4];
             int n = 0;
 #pragma unroll
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
             }
         }
         if (C > 1 && first)
-            for (int w = t; w < words; w += SOLO_T)
+            for (int w = t; w < words; w += T)
                 if ((w & (C - 1)) != rank) vis[w] = dld32(at<C>(s_vis + 4u * w, w & (C - 1)));
         if (t == 0) {
             sm.pub[(s + 2) % 3] = Pub{0, 0, 0, 0};
@@ -465,8 +467,8 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
         for (;;) {
             // a narrow level's columns are dealt to all warps: a warp's time is its chain of instructions
             int width = 32;
-            while (width > 1 && nl <= width / 2 * (SOLO_T / 32)) width >>= 1;
-            for (int g = warp * width; g < nl; g += width * (SOLO_T / 32)) {  // warp-uniform
+            while (width > 1 && nl <= width / 2 * (T / 32)) width >>= 1;
+            for (int g = warp * width; g < nl; g += width * (T / 32)) {  // warp-uniform
                 int beg = 0, deg = 0;
                 unsigned e = 0;
                 if (lane < width && g + lane < nl) {
@@ -552,7 +554,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
         if (eps == 0) break;  // no augmenting path: the matching is maximum (Berge)
         if (phases >= bmd::CARRY_PHASES) carry = false;
         int kept = 0;
-        for (int ow = warp; ow < (int)lay.own_cw; ow += SOLO_T / 32) {
+        for (int ow = warp; ow < (int)lay.own_cw; ow += T / 32) {
             const int w = ow * C + rank, sl = ow * 32 + lane, me = w * 32 + lane;
             if (w >= words) continue;  // warp-uniform
             const unsigned v = vis[w], in_tree = v >> lane & 1u;
@@ -585,8 +587,8 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
         }
         if (lane == 0 && kept) atomicAdd(&sm.mine.cnt, kept);
         __syncthreads();
-        for (int w = t; w < words; w += SOLO_T) srv[w] = 0u;
-        for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += SOLO_T) rcl[w] = 0u;
+        for (int w = t; w < words; w += T) srv[w] = 0u;
+        for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += T) rcl[w] = 0u;
         if (t == 0) {
             if (rank == 0 && bmd::globaltimer() > deadline) sm.mine.flag = -5 /*BM_ERR_TIMEOUT*/;
         }
@@ -598,7 +600,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
     }
     // ---- results: every block its own words
     if (status >= 0) {
-        for (int w = rank + C * warp; w < (nr + 31) >> 5; w += C * (SOLO_T / 32)) {
+        for (int w = rank + C * warp; w < (nr + 31) >> 5; w += C * (T / 32)) {
             const int r = w * 32 + lane;
             if (r < nr) {
                 const int c = rm[r] == SOLO_FREE ? -1 : rm[r];
@@ -606,7 +608,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
                 if (a.rm_out) a.rm_out[r] = c;
             }
         }
-        for (int w = rank + C * warp; w < words; w += C * (SOLO_T / 32)) {
+        for (int w = rank + C * warp; w < words; w += C * (T / 32)) {
             const int c = w * 32 + lane;
             if (c < nc) {
                 const int v = cm[slot_of<C>(c)], r = v == SOLO_FREE ? -1 : v;
@@ -661,8 +663,8 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo(Params p, SoloArgs a, long l
 // rows' states in their owners' shared memory, the columns by degree, columns of
 // more than GREEDY_LIGHT rows a warp each from the block's list.  Adds to the
 // installed matching; |M| goes to the control block and the host's copy.
-template <int C>
-__global__ void __launch_bounds__(SOLO_T, 1) k_solo_greedy(Params p, const int32_t* __restrict__ rdeg, Ctl* h_ctl) {
+template <int C, int T>
+__global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* __restrict__ rdeg, Ctl* h_ctl) {
     using namespace bmd;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ int s_card, s_long;
@@ -675,7 +677,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo_greedy(Params p, const int32
     if (t == 0) s_card = s_long = 0;
     __syncthreads();
     int n = 0;
-    for (int w = rank + C * warp; w < (nr + 31) >> 5; w += C * (SOLO_T / 32)) {
+    for (int w = rank + C * warp; w < (nr + 31) >> 5; w += C * (T / 32)) {
         const int r = w * 32 + lane;
         if (r >= nr) continue;
         const bool is_free = p.rmatch[r] == -1;
@@ -691,7 +693,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo_greedy(Params p, const int32
     const int limit[4] = {0, 2, 8, GREEDY_LIGHT};
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
-        for (unsigned k0 = warp; k0 < (1u << bits); k0 += SOLO_T / 32) {
+        for (unsigned k0 = warp; k0 < (1u << bits); k0 += T / 32) {
             const int own = (int)scatter_bits(k0, bits);
             if (own >= own_tiles) continue;
             const int c = scatter_lane((unsigned)(own * C + rank), lane);
@@ -714,7 +716,7 @@ __global__ void __launch_bounds__(SOLO_T, 1) k_solo_greedy(Params p, const int32
         }
         cluster_sync<C>();
     }
-    for (int k = warp; k < s_long; k += SOLO_T / 32) {  // warp-uniform
+    for (int k = warp; k < s_long; k += T / 32) {  // warp-uniform
         const int c = longs[k];
         if (p.cmatch[c] != -1) continue;
         const int beg = __ldg(&p.col_ptr[c]);

@@ -769,11 +769,11 @@ int grid_for(bm_ctx* ctx, int n) {  // plain launches: enough blocks to fill the
 // Small graphs run on one block or one cluster of 16 blocks (bm_solo.cuh): the default mode with the
 // launch geometry and the barrier limit left to the library.  Returns the blocks, 0 for other graphs.
 // Cheap matching + search, us, on the grid / one block / 16 blocks (one GB300): 100 rows 137 / 66 / -;
-// 1,000 rows (2.8 k entries) 166 / 92 / 95; 3,000 rows (9 k) 240 / 133 / 127; 10,000 rows (45 k)
-// 374 / 372 / 223; 20,000 rows 344 / - / 208; 60,000 rows 463 / - / 391, but 551 / - / 662 for its search
-// from the empty matching, whose levels are wide.
+// 1,000 rows (2.8 k entries) 166 / 82 / 95; 2,000 rows (6 k) - / 134 / 143; 3,000 rows (9.3 k) 240 / 152 /
+// 127; 10,000 rows (45 k) 374 / - / 215; 20,000 rows 344 / - / 205; 60,000 rows 463 / - / 391, but 551 / - /
+// 662 for its search from the empty matching, whose levels are wide.
 constexpr int kSoloBlocks = 16;
-constexpr int64_t kSoloOneBlock = 4096;    // entries up to which one block is faster than 16
+constexpr int64_t kSoloOneBlock = 8192;    // entries up to which one block is faster than 16
 constexpr int32_t kSoloMaxSide = 32768;    // rows and columns up to which 16 blocks are faster than the grid
 constexpr int64_t kSoloMaxEdges = 393216;  // ... and entries (8 MB of L2-resident rows is the grid's)
 
@@ -789,7 +789,7 @@ int solo_cluster(const bm_ctx* ctx) {
 
 void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int C, size_t smem, cudaStream_t st) {
     cfg.gridDim = dim3((unsigned)C);
-    cfg.blockDim = dim3(bms1::SOLO_T);
+    cfg.blockDim = dim3(C == 1 ? bms1::SOLO_T1 : bms1::SOLO_T);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -815,15 +815,15 @@ int32_t configure_solo(bm_ctx* ctx) {
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bms1::SOLO_SMEM);
         return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     };
-    BM_CUDA(ctx, prepare(bms1::k_solo<1>));
-    BM_CUDA(ctx, prepare(bms1::k_solo<kSoloBlocks>));
-    BM_CUDA(ctx, prepare(bms1::k_solo_greedy<1>));
-    BM_CUDA(ctx, prepare(bms1::k_solo_greedy<kSoloBlocks>));
+    BM_CUDA(ctx, prepare(bms1::k_solo<1, bms1::SOLO_T1>));
+    BM_CUDA(ctx, prepare(bms1::k_solo<kSoloBlocks, bms1::SOLO_T>));
+    BM_CUDA(ctx, prepare(bms1::k_solo_greedy<1, bms1::SOLO_T1>));
+    BM_CUDA(ctx, prepare(bms1::k_solo_greedy<kSoloBlocks, bms1::SOLO_T>));
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at[1];
     cluster_config(cfg, at, kSoloBlocks, bms1::SOLO_SMEM, ctx->stream);
     int n = 0;
-    ctx->solo_clusters = cudaOccupancyMaxActiveClusters(&n, bms1::k_solo<kSoloBlocks>, &cfg) == cudaSuccess && n > 0;
+    ctx->solo_clusters = cudaOccupancyMaxActiveClusters(&n, bms1::k_solo<kSoloBlocks, bms1::SOLO_T>, &cfg) == cudaSuccess && n > 0;
     (void)cudaGetLastError();
     ctx->solo_ready = true;
     return BM_OK;
@@ -1106,7 +1106,7 @@ int32_t report(bm_ctx* ctx, bool solo, int32_t* card_out, bm_stats* stats) {
         stats->roots = h.roots;
         if (solo) {
             stats->grid = solo_cluster(ctx);
-            stats->block = bms1::SOLO_T;
+            stats->block = stats->grid == 1 ? bms1::SOLO_T1 : bms1::SOLO_T;
         } else if (ctx->opt.driver == BM_DRIVER_PERSISTENT) {
             stats->grid = ctx->coop_grid[ctx->opt.deterministic ? 2 : ctx->opt.bfs == BM_GPUBFS_WR ? 1 : 0];
             stats->block = ctx->block;
@@ -1130,7 +1130,7 @@ bool solo_match(const bm_ctx* ctx) {
 cudaError_t run_solo_greedy(bm_ctx* ctx) {
     const int C = solo_cluster(ctx);
     const size_t smem = 128 * ((((size_t)ctx->nr + 31) / 32 + C - 1) / C);
-    return launch_cluster(C == 1 ? bms1::k_solo_greedy<1> : bms1::k_solo_greedy<kSoloBlocks>, C, smem, ctx->stream,
+    return launch_cluster(C == 1 ? bms1::k_solo_greedy<1, bms1::SOLO_T1> : bms1::k_solo_greedy<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream,
                           make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl);
 }
 
@@ -1146,7 +1146,7 @@ int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool
     ctx->empty = false;
     const int C = solo_cluster(ctx);
     const size_t smem = bms1::Layout(ctx->nr, ctx->nc, ctx->nnz, C).bytes;
-    BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo<1> : bms1::k_solo<kSoloBlocks>, C, smem, ctx->stream, p, a,
+    BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo<1, bms1::SOLO_T1> : bms1::k_solo<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream, p, a,
                                 (long long)ctx->nnz));
     BM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return report(ctx, true, card_out, stats);

@@ -26,8 +26,8 @@ def hub_graph():
 CASES = {
     "1x1": lambda: csr_from_edges(1, 1, [(0, 0)]),
     "31x33": lambda: synth.uniform_graph(31, 33, 3, seed=1),
-    "4096 entries": lambda: csr_from_edges(1500, 1024, [((7 * c + 31 * k * k) % 1500, c) for c in range(1024) for k in range(4)]),
-    "4097 entries": lambda: csr_from_edges(1500, 1025, [((7 * c + 31 * k * k) % 1500, c) for c in range(1024) for k in range(4)] + [(3, 1024)]),
+    "8192 entries": lambda: csr_from_edges(1500, 1024, [((7 * c + 31 * k * k) % 1500, c) for c in range(1024) for k in range(8)]),
+    "8193 entries": lambda: csr_from_edges(1500, 1025, [((7 * c + 31 * k * k) % 1500, c) for c in range(1024) for k in range(8)] + [(3, 1024)]),
     "few columns": lambda: synth.uniform_graph(30000, 511, 40, seed=2),
     "few rows": lambda: synth.uniform_graph(600, 20000, 5, seed=3),
     "at the side limit": lambda: synth.uniform_graph(32768, 32768, 4, seed=4),
