@@ -107,7 +107,8 @@ struct alignas(128) Ctl {
     int32_t ep_alt;            // the persistent one-endpoint kernel's even phases count their endpoints
                                // here (odd ones in ep_phase), so that each phase's counter can be
                                // cleared during the phase before it
-    int32_t pad1[6];
+    int32_t max_deg;           // CSR check: the longest column
+    int32_t pad1[5];
     long long levels;
     long long max_levels;
     long long cols_expanded;
@@ -606,12 +607,12 @@ __device__ __forceinline__ void step_carry(const Params& p, const int2* q, int t
     const int per = T <= QBUF / 4 ? 4 : QBUF / T;  // entries per thread per pass: at most QBUF a block
     const int walkers = min((n_ep + T - 1) / T, (int)gridDim.x);
     const int me = (int)(blockIdx.x + gridDim.x - walkers) % (int)gridDim.x;
-    for (int base = me * per * T; base < tail; base += gridDim.x * per * T) {  // block-uniform
+    for (long long base = (long long)me * per * T; base < tail; base += (long long)gridDim.x * per * T) {  // block-uniform
         int2 e[4];
         int lv[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int i = base + u * T + (int)threadIdx.x;
+            const long long i = base + u * T + (int)threadIdx.x;
             e[u] = (u < per && i < tail) ? __ldcg(&q[i]) : make_int2(-1, -1);
             if (e[u].x >= 0 && (!idx_ok(p, e[u].x, p.nc) || !idx_ok(p, e[u].y, p.nc))) e[u].x = -1;
         }

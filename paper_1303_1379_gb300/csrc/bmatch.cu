@@ -311,8 +311,13 @@ __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __rest
     const long long nthr = (long long)gridDim.x * blockDim.x;
     bool bad = false;
     if (tid == 0 && (cp[0] != 0 || (long long)cp[nc] != nnz)) bad = true;
-    for (long long c = tid; c < nc; c += nthr)
+    int longest = 0;
+    for (long long c = tid; c < nc; c += nthr) {
+        const int d = cp[c + 1] - cp[c];
         if (cp[c + 1] < cp[c]) bad = true;
+        longest = max(longest, d);
+    }
+    if (longest > bmd::ld_volatile(&ctl->max_deg)) atomicMax(&ctl->max_deg, longest);
     for (long long e = tid; e < nnz; e += nthr) {
         int r = __ldg(&ri[e]);
         if (r < 0 || r >= nr) bad = true;
@@ -422,8 +427,22 @@ struct GreedyLists {
     int32_t* count;   // [2] their lengths, zero before the light pass
 };
 
-// state[r] from the matching the passes start from (rdeg may be state itself).
-__global__ void k_greedy_state(int nr, const int32_t* __restrict__ rm, const int32_t* rdeg, int32_t* state) {
+// Adds the block's n to *dst with one atomic.
+__device__ __forceinline__ void block_count(int32_t* dst, int n) {
+    __shared__ int s_n;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    n = __reduce_add_sync(bmd::FULL, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(&s_n, n);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_n) atomicAdd(dst, s_n);
+}
+
+// state[r] from the matching the passes start from (rdeg may be state itself).  clear (nullable): the control
+// block's words that the passes and the caller use go to zero (in place of a fill of its own before).
+__global__ void k_greedy_state(int nr, const int32_t* __restrict__ rm, const int32_t* rdeg, int32_t* state, Ctl* clear) {
+    if (clear && blockIdx.x == 0 && threadIdx.x == 0)
+        clear->qcnt[0] = clear->qcnt[1] = clear->card = clear->err = clear->searches = 0;
     for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nr; r += gridDim.x * blockDim.x)
         state[r] = rm[r] == -1 ? rdeg[r] : GREEDY_TAKEN;
 }
@@ -431,9 +450,10 @@ __global__ void k_greedy_state(int nr, const int32_t* __restrict__ rm, const int
 // Columns of LO < degree <= HI; LISTS: also lists the columns of the later passes.
 template <int LO, int HI, bool LISTS>
 __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int32_t* __restrict__ ri,
-                               int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl, const Ctl* ctl) {
+                               int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl, Ctl* ctl) {
     // after an asynchronous CSR check on the same stream: an invalid CSR is not read
-    if (ctl && bmd::ld_volatile(&ctl->err) != 0) return;
+    if (bmd::ld_volatile(&ctl->err) != 0) return;
+    int n = 0;  // columns this thread matched (LISTS: and those that were)
     constexpr int U = HI < 4 ? HI : 4;
     const unsigned tiles = ((unsigned)nc + 31) >> 5;
     const int bits = tiles > 1 ? 32 - __clz(tiles - 1) : 0;  // 2^bits >= tiles
@@ -445,8 +465,12 @@ __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int
         if (c >= nc) continue;
         const int beg = __ldg(&cp[c]);
         const int deg = __ldg(&cp[c + 1]) - beg;
-        if (LISTS ? deg <= LO : (deg <= LO || deg > HI)) continue;
-        if (cm[c] != -1) continue;
+        if (!LISTS && (deg <= LO || deg > HI)) continue;
+        if (cm[c] != -1) {
+            n += LISTS;
+            continue;
+        }
+        if (LISTS && deg <= LO) continue;
         if (LISTS) {
             if (deg > GREEDY_MEDIUM) bmd::push(gl.heavy, 0, &gl.count[1], c);
             else if (deg > GREEDY_LIGHT) bmd::push(gl.medium, 0, &gl.count[0], c);
@@ -460,15 +484,18 @@ __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int
             if (atomicCAS(&state[r], seen, GREEDY_TAKEN) == seen) {
                 rm[r] = c;
                 cm[c] = r;
+                ++n;
                 break;
             }
         }
     }
+    block_count(&ctl->card, n);
 }
 
 __global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri, int32_t* state,
-                                int32_t* rm, int32_t* cm, GreedyLists gl, const Ctl* ctl) {
-    if (ctl && bmd::ld_volatile(&ctl->err) != 0) return;
+                                int32_t* rm, int32_t* cm, GreedyLists gl, Ctl* ctl) {
+    if (bmd::ld_volatile(&ctl->err) != 0) return;
+    int won = 0;
     const int lane = threadIdx.x & 31;
     const int n = gl.count[0];
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -482,14 +509,16 @@ __global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* _
         if (r >= 0 && lane == 0) {
             rm[r] = hc;
             cm[hc] = r;
+            ++won;
         }
     }
+    block_count(&ctl->card, won);
 }
 
 __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri,
                                                        int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl,
-                                                       const Ctl* ctl) {
-    if (ctl && bmd::ld_volatile(&ctl->err) != 0) return;
+                                                       Ctl* ctl) {
+    if (bmd::ld_volatile(&ctl->err) != 0) return;
     __shared__ int s_pos, s_done;
     const int T = blockDim.x, t = threadIdx.x;
     const int n = gl.count[1];
@@ -529,6 +558,7 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
                     if (atomicCAS(&state[rr], seen, GREEDY_TAKEN) == seen) {
                         rm[rr] = hc;
                         cm[hc] = rr;
+                        atomicAdd(&ctl->card, 1);
                         s_done = 1;
                     }
                     s_pos = 0x7fffffff;
@@ -552,18 +582,21 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
 // The cheap matching (Section 4) on the device: columns by degree, shortest
 // lists first.  `rdeg` holds the rows' entry counts, `state` is scratch of nr
 // int32 (it may be rdeg, whose counts are then lost), `lists` of 2 x nc int32
-// (the context's queue, free before a match) and `count` two int32 cleared
-// beforehand.
-void launch_greedy(int nr, int nc, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, const Ctl* ctl,
-                   const int32_t* rdeg, int32_t* state, int32_t* lists, int32_t* count, int grid, int block,
+// (the context's queue, free before a match); their lengths are counted in the
+// first two queue counters, |M| in ctl->card.  clear: the passes' first launch
+// zeroes those words and the error (otherwise they are zero beforehand, and an
+// error set there stops the passes).  Passes that no column of up to max_deg
+// rows needs are not launched: a launch costs a call about 5 us.
+void launch_greedy(int nr, int nc, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, Ctl* ctl, bool clear,
+                   int max_deg, const int32_t* rdeg, int32_t* state, int32_t* lists, int grid, int block,
                    cudaStream_t st) {
-    const GreedyLists gl{lists, lists + nc, count};
-    k_greedy_state<<<grid, block, 0, st>>>(nr, rm, rdeg, state);
+    const GreedyLists gl{lists, lists + nc, &ctl->qcnt[0]};
+    k_greedy_state<<<grid, block, 0, st>>>(nr, rm, rdeg, state, clear ? ctl : nullptr);
     k_greedy_light<0, 2, true><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    k_greedy_medium<<<grid, block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
-    k_greedy_heavy<<<grid, block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
+    if (max_deg > 2) k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    if (max_deg > 8) k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    if (max_deg > GREEDY_LIGHT) k_greedy_medium<<<grid, block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
+    if (max_deg > GREEDY_MEDIUM) k_greedy_heavy<<<grid, block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
 }
 
 // The cheap matching of the deterministic option over the whole GPU (one
@@ -696,6 +729,7 @@ struct bm_ctx {
     bool owns_csr = false;
     bool csr_ready = false;
     bool empty = false;  // the installed matching is known to be empty
+    int32_t max_deg = 0x7fffffff;  // the longest column, where the host has read it
     cudaStream_t stream = nullptr;
     bm_options opt{};
     void* arena = nullptr;  // one device allocation for everything the context owns
@@ -1037,9 +1071,9 @@ int32_t run(bm_ctx* ctx, bool bfs_only) {
     Params p = make_params(ctx, bfs_only);
     if (!bfs_only && starts_cheap(ctx)) {
         // (its list counters are two of the queue counters, which the matching kernel needs at zero)
-        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, ctx->rdeg,
-                      ctx->endpoints, (int32_t*)ctx->queue, &ctx->ctl->qcnt[0], grid_for(ctx, ctx->nc), ctx->block,
-                      ctx->stream);
+        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, false,
+                      ctx->max_deg, ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_for(ctx, ctx->nc),
+                      ctx->block, ctx->stream);
         BM_CUDA(ctx, cudaGetLastError());
         BM_CUDA(ctx, cudaMemsetAsync(&ctx->ctl->qcnt[0], 0, 2 * sizeof(int32_t), ctx->stream));
         p.pre = 1;
@@ -1300,6 +1334,7 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
         if (!rc) rc = sync_ctl(ctx);
         if (!rc && ctx->h_ctl->err) rc = ctx->h_ctl->err;
         if (rc) { bm_destroy(ctx); return rc; }
+        ctx->max_deg = ctx->h_ctl->max_deg;
         ctx->csr_ready = true;
     } else {
         rc = sync_ctl(ctx);
@@ -1331,6 +1366,7 @@ int32_t bm_upload_csr(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     if (!rc) rc = sync_ctl(ctx);
     if (rc) return rc;
     if (ctx->h_ctl->err) { ctx->csr_ready = false; return ctx->h_ctl->err; }
+    ctx->max_deg = ctx->h_ctl->max_deg;
     ctx->csr_ready = true;
     return BM_OK;
 }
@@ -1347,7 +1383,7 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         if (card_out) *card_out = ctx->h_ctl->card;
         return BM_OK;
     }
-    BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
+    if (!ctx->nc || ctx->opt.deterministic) BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     if (ctx->nc && ctx->opt.deterministic) {
         // proposal rounds: the same matching on every run and launch geometry
         int32_t rc = ensure_det_arena(ctx);
@@ -1360,10 +1396,8 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
         BM_CUDA(ctx, cudaGetLastError());
     } else if (ctx->nc) {
-        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, nullptr, ctx->rdeg,
-                      ctx->endpoints, (int32_t*)ctx->queue, &ctx->ctl->qcnt[0], grid_for(ctx, ctx->nc), ctx->block, st);
-        BM_CUDA(ctx, cudaGetLastError());
-        k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
+        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->max_deg,
+                      ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_for(ctx, ctx->nc), ctx->block, st);
         BM_CUDA(ctx, cudaGetLastError());
     }
     int32_t rc = sync_ctl(ctx);
@@ -1487,6 +1521,7 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     k_check_matching<<<grid_for(ctx, ctx->nr > ctx->nc ? ctx->nr : ctx->nc), ctx->block, 0, st>>>(ctx->nr, ctx->nc, ctx->rmatch, ctx->cmatch, ctx->ctl);
     BM_CUDA(ctx, cudaGetLastError());
     ctx->csr_ready = true;
+    ctx->max_deg = 0x7fffffff;  // (not read back)
     if (ctx->opt.driver == BM_DRIVER_HOST) {
         rc = sync_ctl(ctx);
         if (rc) return rc;
@@ -1807,8 +1842,8 @@ int32_t bmi::enqueue_match(bmd::Params p, long long nnz, bool wr, int greedy, cu
     } else if (greedy) {
         // the cheap matching counts its lists in the control block's first two queue
         // counters, which the matching kernel needs at zero
-        launch_greedy(p.nr, p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, rdeg, rdeg, (int32_t*)p.queue,
-                      &p.ctl->qcnt[0], grid_of(p.nc), B, st);
+        launch_greedy(p.nr, p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, false, 0x7fffffff, rdeg, rdeg,
+                      (int32_t*)p.queue, grid_of(p.nc), B, st);
         if (cudaMemsetAsync(&p.ctl->qcnt[0], 0, 2 * sizeof(int32_t), st) != cudaSuccess) {
             (void)cudaGetLastError();
             return BM_ERR_CUDA;
