@@ -1904,66 +1904,73 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
 // The cheap matching of the deterministic option, by one block: rounds in
 // which every unmatched column proposes to the first unmatched row of its
 // list and every proposed row takes the smallest proposer (atomicMin in
-// ekey[r]); until a round without proposals.  Columns of more than 32 rows
-// look for their row a warp at a time (32 rows per step, a ballot of the free
-// ones), from a list in the queue buffer; the others a thread each.
-// Scratch: level (position in the column's list), root (the row proposed to,
-// -1 none); ekey must be all ones before and is again after.
-template <bool NC>
+// ekey[r]); until a round without proposals.  A column that found no row has
+// none left, so a round takes only the columns that proposed in the one before
+// (lists in dkey's space, which is not in use yet).  Columns of more than 32
+// rows look for their row a warp at a time (32 rows per step, a ballot of the
+// free ones), from a list in the queue buffer; the others a thread each.
+// Scratch: level (position in the column's list), root (the row proposed to);
+// ekey must be all ones before and is again after.
+// ROWS: p.vis (shared memory) has one bit per matched row, so that the scans
+// read no matches.
+template <bool NC, bool ROWS>
 __device__ __forceinline__ void block_greedy_rounds(const Params& p, Smem& sm) {
     const int T = blockDim.x, t = threadIdx.x, nc = p.nc;
     const int lane = t & 31, warp = t >> 5, nwarps = (T + 31) >> 5;
     int32_t* longs = (int32_t*)p.queue;
-    if (t == 0) sm.tile = 0;
+    int32_t* list = (int32_t*)p.dkey;  // proposers of a round
+    int32_t* other = list + nc;
+    auto is_free = [&](int r) {
+        if (ROWS) return !sb_test(p.vis, r);
+        return __ldcg(&p.rmatch[r]) == -1;
+    };
+    auto propose = [&](int c, int want, int32_t* to) {
+        __stcg(&p.root[c], want);
+        atomicMin(&p.ekey[want], (unsigned long long)(unsigned)c);
+        to[atomicAdd(&sm.qn, 1)] = c;
+    };
+    auto search_short = [&](int c, int pos, int end, int32_t* to) {
+        while (pos < end) {  // 4 rows per step, their matches in flight together
+            int r[4];
+            bool f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) r[u] = pos + u < end ? ld_csr<NC>(&p.row_idx[pos + u]) : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) f[u] = r[u] >= 0 && idx_ok(p, r[u], p.nr) && is_free(r[u]);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (f[u]) {
+                    __stcg(&p.level[c], pos + u);
+                    propose(c, r[u], to);
+                    return;
+                }
+            pos += 4;
+        }
+    };
+    if (t == 0) sm.tile = sm.qn = 0;
     __syncthreads();
-    for (int c = t; c < nc; c += T) {
-        const int b = ld_csr<NC>(&p.col_ptr[c]);
-        __stcg(&p.level[c], b);
-        if (ld_csr<NC>(&p.col_ptr[c + 1]) - b > 32) longs[atomicAdd(&sm.tile, 1)] = c;
+    for (int c = t; c < nc; c += T) {  // the first round's short lists, and the list of the long ones
+        const int b = ld_csr<NC>(&p.col_ptr[c]), e = ld_csr<NC>(&p.col_ptr[c + 1]);
+        if (e - b > 32) {
+            __stcg(&p.level[c], b);
+            longs[atomicAdd(&sm.tile, 1)] = c;
+        } else if (__ldcg(&p.cmatch[c]) == -1) {
+            search_short(c, b, e, list);
+        }
     }
     __syncthreads();
     const int nlong = sm.tile;
     for (int round = 0; round <= nc; ++round) {
-        if (t == 0) sm.ok = 0;
-        __syncthreads();
-        bool any = false;
-        for (int c = t; c < nc; c += T) {  // short lists: a thread each
-            const int end = ld_csr<NC>(&p.col_ptr[c + 1]);
-            if (end - ld_csr<NC>(&p.col_ptr[c]) > 32) continue;
-            int want = -1;
-            if (__ldcg(&p.cmatch[c]) == -1) {
-                int pos = __ldcg(&p.level[c]);
-                while (pos < end) {  // 4 rows per step, their matches in flight together
-                    int r[4], m[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) r[u] = pos + u < end ? ld_csr<NC>(&p.row_idx[pos + u]) : -1;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) m[u] = (r[u] >= 0 && idx_ok(p, r[u], p.nr)) ? __ldcg(&p.rmatch[r[u]]) : 0;
-                    int k = 0;
-                    while (k < 4 && r[k] >= 0 && m[k] != -1) ++k;
-                    if (k < 4 && r[k] >= 0) { pos += k; want = r[k]; break; }
-                    pos += 4;
-                }
-                if (pos > end) pos = end;
-                __stcg(&p.level[c], pos);
-                if (want >= 0) {
-                    atomicMin(&p.ekey[want], (unsigned long long)(unsigned)c);
-                    any = true;
-                }
-            }
-            __stcg(&p.root[c], want);
-        }
         for (int k = warp; k < nlong; k += nwarps) {  // long lists: a warp each (warp-uniform)
             const int c = __ldcg(&longs[k]);
             if (!idx_ok(p, c, nc)) continue;
-            int want = -1;
             if (__ldcg(&p.cmatch[c]) == -1) {
                 const int end = ld_csr<NC>(&p.col_ptr[c + 1]);
-                int pos = __ldcg(&p.level[c]);
+                int pos = __ldcg(&p.level[c]), want = -1;
                 while (pos < end) {
                     const int r = pos + lane < end ? ld_csr<NC>(&p.row_idx[pos + lane]) : -1;
-                    const int m = (r >= 0 && idx_ok(p, r, p.nr)) ? __ldcg(&p.rmatch[r]) : 0;
-                    const unsigned free_rows = __ballot_sync(FULL, r >= 0 && m == -1);
+                    const unsigned free_rows =
+                        __ballot_sync(FULL, r >= 0 && idx_ok(p, r, p.nr) && is_free(r));
                     if (free_rows) {
                         const int k0 = __ffs(free_rows) - 1;
                         pos += k0;
@@ -1972,33 +1979,38 @@ __device__ __forceinline__ void block_greedy_rounds(const Params& p, Smem& sm) {
                     }
                     pos += 32;
                 }
-                if (pos > end) pos = end;
                 if (lane == 0) {
-                    __stcg(&p.level[c], pos);
-                    if (want >= 0) atomicMin(&p.ekey[want], (unsigned long long)(unsigned)c);
+                    __stcg(&p.level[c], pos < end ? pos : end);
+                    if (want >= 0) propose(c, want, list);
                 }
-                if (want >= 0) any = true;
             }
-            if (lane == 0) __stcg(&p.root[c], want);
         }
-        if (any) sm.ok = 1;
         __syncthreads();
-        const bool more = sm.ok != 0;
-        for (int c = t; c < nc; c += T) {
-            const int r = __ldcg(&p.root[c]);
-            if (r >= 0 && __ldcg(&p.ekey[r]) == (unsigned long long)(unsigned)c) {
+        const int n = sm.qn;
+        if (n == 0) break;
+        for (int i = t; i < n; i += T) {
+            const int c = __ldcg(&list[i]), r = __ldcg(&p.root[c]);
+            if (__ldcg(&p.ekey[r]) == (unsigned long long)(unsigned)c) {
                 __stcg(&p.rmatch[r], c);
                 __stcg(&p.cmatch[c], r);
+                if (ROWS) atomicOr(&p.vis[r >> 5], 1u << (r & 31));
             }
         }
         __syncthreads();
-        for (int c = t; c < nc; c += T) {
-            const int r = __ldcg(&p.root[c]);
-            if (r >= 0) __stcg(&p.ekey[r], DKEY_NONE);
-        }
+        if (t == 0) sm.qn = 0;
+        for (int i = t; i < n; i += T) __stcg(&p.ekey[__ldcg(&p.root[__ldcg(&list[i])])], DKEY_NONE);
         __syncthreads();
-        if (!more) break;
+        for (int i = t; i < n; i += T) {  // the next round's short lists
+            const int c = __ldcg(&list[i]);
+            if (__ldcg(&p.cmatch[c]) != -1) continue;
+            const int e = ld_csr<NC>(&p.col_ptr[c + 1]);
+            if (e - ld_csr<NC>(&p.col_ptr[c]) <= 32) search_short(c, __ldcg(&p.level[c]), e, other);
+        }
+        int32_t* const x = list;
+        list = other;
+        other = x;
     }
+    __syncthreads();
 }
 
 // The whole method on one graph by one block with the deterministic option's
@@ -2018,16 +2030,30 @@ __device__ int block_match_graph_det(const Params& p, int greedy, Smem& sm, Coun
     const int t = threadIdx.x;
     const int nr = p.nr, nc = p.nc;
     if (t == 0) sm.ok = 0;
-    // ---- rows whose column does not point back are unmatched; every key "none"
-    for (int r = t; r < nr; r += T) {
-        const int m = __ldcg(&p.rmatch[r]);
-        if (m != -1 && (m < 0 || m >= nc || __ldcg(&p.cmatch[m]) != r)) __stcg(&p.rmatch[r], -1);
-        __stcg(&p.ekey[r], DKEY_NONE);
+    // ---- rows whose column does not point back are unmatched; every key "none"; a warp takes 32 consecutive
+    // rows and, with marks for the rounds (SB, as far as the bitmap goes), writes their word
+    const bool rows_sb = SB && nr <= SB_MAX_COLS;
+    for (int r0 = t & ~31; r0 < nr; r0 += T) {  // warp-uniform: blockDim is a multiple of 32
+        const int r = r0 + (t & 31);
+        int m = -1;
+        if (r < nr) {
+            m = __ldcg(&p.rmatch[r]);
+            if (m != -1 && (m < 0 || m >= nc || __ldcg(&p.cmatch[m]) != r)) {
+                __stcg(&p.rmatch[r], -1);
+                m = -1;
+            }
+            __stcg(&p.ekey[r], DKEY_NONE);
+        }
+        const unsigned w = __ballot_sync(FULL, m != -1);
+        if (rows_sb && (t & 31) == 0) p.vis[r0 >> 5] = w;
+    }
+    __syncthreads();
+    if (greedy) {
+        if (rows_sb) block_greedy_rounds<NC, true>(p, sm);
+        else block_greedy_rounds<NC, false>(p, sm);
     }
     for (int c = t; c < nc; c += T) __stcg(&p.dkey[c], DKEY_NONE);
     __syncthreads();
-    if (greedy) block_greedy_rounds<NC>(p, sm);
-    if (t == 0) sm.ok = 0;  // the rounds used it as their flag; from here it holds Alternate's errors
     const int max_phases = (nr < nc ? nr : nc) + 2;
     int phases = 0, card = 0, status = 0;
     long long levels_total = 0, eps_total = 0, ins_total = 0;
