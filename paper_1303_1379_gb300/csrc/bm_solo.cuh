@@ -522,7 +522,10 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
             wins = __reduce_add_sync(FULL, wins);
             if (lane == 0 && wins) atomicAdd(&sm.mine.cnt, wins);
             wins = 0;
+            // the launch's limit, at every eighth level: a phase of a long path is thousands of them
+            if (leader && (level & 7) == 0 && bmd::globaltimer() > deadline) sm.mine.flag = -5 /*BM_ERR_TIMEOUT*/;
             end_step(false);
+            if (flag != 0) break;  // the same in every block
             ++level;
             eps += sum_eps;
             if (leader) {
@@ -537,6 +540,10 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
             if (carry && eps > 0 && phases <= bmd::CUT_PHASES && level >= bmd::CUT_MIN && level <= bmd::CUT_MAX &&
                 sum_cnt * bmd::CUT_RATIO <= tail)
                 break;
+        }
+        if (flag != 0) {
+            status = flag;
+            break;
         }
         if (leader) {
             SoloStats& g = sm.st;
@@ -589,9 +596,6 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         __syncthreads();
         for (int w = t; w < words; w += T) srv[w] = 0u;
         for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += T) rcl[w] = 0u;
-        if (t == 0) {
-            if (rank == 0 && bmd::globaltimer() > deadline) sm.mine.flag = -5 /*BM_ERR_TIMEOUT*/;
-        }
         end_step(true);
         n_front = sum_cnt;
         status = flag;
