@@ -88,7 +88,8 @@ typedef struct bm_options {
                                 number of endpoints per root, the root slot set to L0-2
                                 (Algorithm 4 as printed)                                   */
     int32_t max_phases;    /* 0 = no limit besides the safety cap min(n_rows,n_cols)+2;
-                              > 0 = stop after that many phases with BM_INCOMPLETE          */
+                              > 0 = stop after that many phases with BM_INCOMPLETE (each then
+                              searches from its roots and to its end)                       */
     int32_t block_size;    /* threads per block, 0 = default (512; a batch whose largest graph sets
                               its time: 1024); multiple of 32, <= 1024 */
     int32_t blocks_per_sm; /* 0 = as many as fit (capped at 2 x 1024 threads per SM)        */

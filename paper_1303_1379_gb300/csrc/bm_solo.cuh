@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         }
         initial = 0;
     }
-    bool carry = true;
+    bool carry = p.phase_limit_is_error != 0;  // (as k_match: not under a caller's phase limit)
     int wins = 0;
 
     // Visits SOLO_U x 32 edges: lane's rows r (own < 0: none) of columns ent >> 16 of root ent & 0xffff.  The

@@ -75,7 +75,9 @@ __global__ void __launch_bounds__(1024, 1) k_match(Params p) {
     int n_roots = 0;
     int n_front = 0;  // entries of the phase's first queue segment: its roots, and the trees carried over
     int iso_free = 0;
-    bool carry = RV && !DET && incr && p.mode == 0;  // trees are carried over to the next phase (see below)
+    // trees are carried over to the next phase, and phases cut (bm_device.cuh, CARRY_PHASES); not under a caller's
+    // limit on the phases, which counts whole ones: a cut phase leaves paths to the next that it would have found
+    bool carry = RV && !DET && incr && p.mode == 0 && p.phase_limit_is_error;
     int no_roots = 0;  // the loop ended because no column was left to search from
     if (ld_volatile(&ctl->err) != 0) goto out;  // input validation failed before launch
     {

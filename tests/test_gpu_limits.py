@@ -46,3 +46,37 @@ def test_time_limit_ends_a_small_graph_within_a_phase(n, limit):
     with bmatch.Matcher(g.n_rows, g.n_cols, g.nnz, cp, ri) as m:  # the GPU and a new context are fine
         res = m.match_from(d_rm, d_cm)
         assert res.card == n - 1 and res.stats["max_levels_in_phase"] == n and res.stats["grid"] in (1, 16)
+
+
+@pytest.mark.parametrize("block", [0, 512])  # one cluster, the grid
+def test_a_limited_phase_is_a_whole_phase(block):
+    """3,000 paths of three levels and 40 of twelve, all apart: one whole phase finds every one, however narrow its
+    last levels are."""
+    g, rm, cm = chains([3] * 3000 + [12] * 40)
+    cp, ri = to_dev(g)
+    with bmatch.Matcher(g.n_rows, g.n_cols, g.nnz, cp, ri, max_phases=1, block_size=block) as m:
+        m.set_matching(torch.from_numpy(rm).cuda(), torch.from_numpy(cm).cuda())
+        res = m.match(allow_incomplete=True)
+        levels, ends, _, _ = m.phase_profile()
+    assert res.card == g.n_cols and res.stats["initial_card"] == g.n_cols - 3040
+    assert levels.tolist() == [12] and ends.tolist() == [3040]
+
+
+@pytest.mark.parametrize("block", [0, 512])
+@pytest.mark.parametrize("phases", [1, 2])
+def test_limited_phases_from_the_empty_matching(block, phases):
+    """The first phase from nothing is one level, with or without the cheap matching's kernels running it: it leaves
+    a maximal matching, and no more than that counts as done."""
+    rng = np.random.default_rng(phases)
+    n = 3000
+    g = csr_from_edges(n, n, [(int(r), c) for c in range(n) for r in rng.integers(0, n, 3)])
+    cp, ri = to_dev(g)
+    rm = torch.empty(n, dtype=torch.int32, device="cuda")
+    cm = torch.empty(n, dtype=torch.int32, device="cuda")
+    with bmatch.Matcher(n, n, g.nnz, cp, ri, max_phases=phases, block_size=block) as m:
+        res = m.match(rm, cm, allow_incomplete=True)
+        levels, ends, _, _ = m.phase_profile()
+    assert len(levels) == phases and levels[0] == 1 and ends.sum() == res.card < oracle_max(g)
+    rm, cm = rm.cpu().numpy(), cm.cpu().numpy()
+    assert np.all(rm[g.row_idx[np.repeat(cm < 0, np.diff(g.col_ptr))]] >= 0)
+    assert res.status == bmatch.BM_INCOMPLETE
