@@ -1,0 +1,53 @@
+"""The cheap matching on graphs of extreme shapes: few columns of many rows and
+the reverse, single degree classes, rows that all columns list, rows whose
+entry counts share a slot, diagonals, hubs."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1303_1379_gb300 import bmatch, synth
+
+from helpers import oracle_max, to_dev
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def regular(nr, nc, k, seed=0):
+    """nc columns of k different rows each."""
+    rng = np.random.default_rng(seed)
+    rows = np.array([rng.choice(nr, k, replace=False) for _ in range(nc)], np.int32)
+    return synth.Graph(nr, nc, (np.arange(nc + 1) * k).astype(np.int32), rows.reshape(-1).copy(), "regular")
+
+
+def from_lists(nr, lists):
+    ptr = np.concatenate([[0], np.cumsum([len(x) for x in lists])]).astype(np.int32)
+    return synth.Graph(nr, len(lists), ptr, np.concatenate(lists).astype(np.int32), "lists")
+
+
+def greedy(g, start=None, first=None, **options):
+    """bm_greedy's (rmatch, cmatch) from `start`; checks that it is valid, maximal and keeps the start."""
+    cp, ri = to_dev(g)
+    rm = torch.empty(g.n_rows, dtype=torch.int32, device="cuda")
+    cm = torch.empty(g.n_cols, dtype=torch.int32, device="cuda")
+    with bmatch.Matcher(g.n_rows, g.n_cols, g.nnz, cp, ri, **options) as m:
+        if first:
+            first(m)
+        m.set_matching()
+        card = m.greedy()
+        m.get_matching(rm, cm)
+        res = m.match()
+    rm, cm = rm.cpu().numpy(), cm.cpu().numpy()
+    assert oracle.validate(g.n_rows, g.n_cols, g.col_ptr, g.row_idx, rm, cm) == (0, card)
+    assert np.all(rm[g.row_idx[np.repeat(cm < 0, np.diff(g.col_ptr))]] >= 0)
+    assert res.card == oracle_max(g)
+    return rm, cm
+
+
+SHAPES = [(100000, 10, 5000), (40000, 300, 300), (33000, 1, 3000), (10, 40000, 3), (600, 40000, 30), (3000, 3000, 300)]
+
+
+@pytest.mark.parametrize("shape", SHAPES, ids=str)
+@pytest.mark.parametrize("block", [0, 64])
+def test_cheap_matching_of_few_columns_or_few_rows(shape, block):
+    greedy(regular(*shape), block_size=block)
