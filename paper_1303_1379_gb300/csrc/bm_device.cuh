@@ -107,7 +107,7 @@ struct alignas(128) Ctl {
     int32_t ep_alt;            // the persistent one-endpoint kernel's even phases count their endpoints
                                // here (odd ones in ep_phase), so that each phase's counter can be
                                // cleared during the phase before it
-    int32_t max_deg;           // CSR check: the longest column
+    int32_t classes;           // CSR check: the degree classes that some column is of (greedy_class)
     int32_t pad1[5];
     long long levels;
     long long max_levels;

@@ -317,6 +317,12 @@ __global__ void __launch_bounds__(1024) k_release(Params p, int n_ep) {
 }
 
 // ---- input checks, greedy, fills
+// The passes of the cheap matching that a column of d rows needs, one bit each (launch_greedy).
+enum : int { CLS_2 = 1, CLS_8 = 2, CLS_LIGHT = 4, CLS_MEDIUM = 8, CLS_HEAVY = 16, CLS_ALL = 31 };
+__device__ __forceinline__ int greedy_class(int d) {
+    return d <= 2 ? CLS_2 : d <= 8 ? CLS_8 : d <= bmd::GREEDY_LIGHT ? CLS_LIGHT : d <= bmd::GREEDY_MEDIUM ? CLS_MEDIUM : CLS_HEAVY;
+}
+
 // rdeg (nullable, zero before): every row's number of entries, counted on the way for
 // the cheap matching.
 __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __restrict__ cp,
@@ -325,13 +331,14 @@ __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __rest
     const long long nthr = (long long)gridDim.x * blockDim.x;
     bool bad = false;
     if (tid == 0 && (cp[0] != 0 || (long long)cp[nc] != nnz)) bad = true;
-    int longest = 0;
+    int classes = 0;
     for (long long c = tid; c < nc; c += nthr) {
-        const int d = cp[c + 1] - cp[c];
-        if (cp[c + 1] < cp[c]) bad = true;
-        longest = max(longest, d);
+        const int b = cp[c], e = cp[c + 1];
+        if (e < b) bad = true;
+        else classes |= greedy_class(e - b);
     }
-    if (longest > bmd::ld_volatile(&ctl->max_deg)) atomicMax(&ctl->max_deg, longest);
+    classes = __reduce_or_sync(bmd::FULL, classes);
+    if ((threadIdx.x & 31) == 0 && (classes & ~bmd::ld_volatile(&ctl->classes))) atomicOr(&ctl->classes, classes);
     for (long long e = tid; e < nnz; e += nthr) {
         int r = __ldg(&ri[e]);
         if (r < 0 || r >= nr) bad = true;
@@ -599,8 +606,9 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
 // (the context's queue, free before a match); their lengths are counted in the
 // first two queue counters, |M| in ctl->card.  clear: the passes' first launch
 // zeroes those words and the error (otherwise they are zero beforehand, and an
-// error set there stops the passes).  Passes that no column of up to max_deg
-// rows needs are not launched: a launch costs a call about 5 us.  Each launch
+// error set there stops the passes).  Passes that no column needs (classes, from
+// the CSR check; the first one lists and counts, so it always runs) are not
+// launched: a launch costs a call about 5 us.  Each launch
 // has as many blocks as its own work fills (cap: what the GPU holds): rows for
 // the states, columns for the light passes, and a warp or a block for every
 // column that may be listed for the other two (blocks beyond the lists end at
@@ -608,17 +616,17 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
 // ran on a block or two (10 columns of 5,000 of 100,000 rows 135 -> 36 us, 1,000
 // columns of 300 of 100,000 rows 127 -> 37 us).
 void launch_greedy(int nr, int nc, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, Ctl* ctl, bool clear,
-                   int max_deg, const int32_t* rdeg, int32_t* state, int32_t* lists, int cap, int block,
+                   int classes, const int32_t* rdeg, int32_t* state, int32_t* lists, int cap, int block,
                    cudaStream_t st) {
     const GreedyLists gl{lists, lists + nc, &ctl->qcnt[0]};
     auto blocks = [&](long long threads) { return (int)std::max(1LL, std::min((threads + block - 1) / block, (long long)cap)); };
     const int grid = blocks(nc);
     k_greedy_state<<<blocks(nr), block, 0, st>>>(nr, rm, rdeg, state, clear ? ctl : nullptr);
     k_greedy_light<0, 2, true><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    if (max_deg > 2) k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    if (max_deg > 8) k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    if (max_deg > GREEDY_LIGHT) k_greedy_medium<<<blocks(32LL * nc), block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
-    if (max_deg > GREEDY_MEDIUM)
+    if (classes & CLS_8) k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    if (classes & CLS_LIGHT) k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
+    if (classes & CLS_MEDIUM) k_greedy_medium<<<blocks(32LL * nc), block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
+    if (classes & CLS_HEAVY)
         k_greedy_heavy<<<blocks((long long)block * nc), block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
 }
 
@@ -752,7 +760,7 @@ struct bm_ctx {
     bool owns_csr = false;
     bool csr_ready = false;
     bool empty = false;  // the installed matching is known to be empty
-    int32_t max_deg = 0x7fffffff;  // the longest column, where the host has read it
+    int32_t classes = CLS_ALL;  // column classes that exist, where the host has read them
     cudaStream_t stream = nullptr;
     bm_options opt{};
     void* arena = nullptr;  // one device allocation for everything the context owns
@@ -1103,7 +1111,7 @@ int32_t run(bm_ctx* ctx, bool bfs_only) {
     if (!bfs_only && starts_cheap(ctx)) {
         // (its list counters are two of the queue counters, which the matching kernel needs at zero)
         launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, false,
-                      ctx->max_deg, ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, ctx->stream);
+                      ctx->classes, ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, ctx->stream);
         BM_CUDA(ctx, cudaGetLastError());
         BM_CUDA(ctx, cudaMemsetAsync(&ctx->ctl->qcnt[0], 0, 2 * sizeof(int32_t), ctx->stream));
         p.pre = 1;
@@ -1364,7 +1372,7 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
         if (!rc) rc = sync_ctl(ctx);
         if (!rc && ctx->h_ctl->err) rc = ctx->h_ctl->err;
         if (rc) { bm_destroy(ctx); return rc; }
-        ctx->max_deg = ctx->h_ctl->max_deg;
+        ctx->classes = ctx->h_ctl->classes;
         ctx->csr_ready = true;
     } else {
         rc = sync_ctl(ctx);
@@ -1396,7 +1404,7 @@ int32_t bm_upload_csr(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     if (!rc) rc = sync_ctl(ctx);
     if (rc) return rc;
     if (ctx->h_ctl->err) { ctx->csr_ready = false; return ctx->h_ctl->err; }
-    ctx->max_deg = ctx->h_ctl->max_deg;
+    ctx->classes = ctx->h_ctl->classes;
     ctx->csr_ready = true;
     return BM_OK;
 }
@@ -1426,7 +1434,7 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
         BM_CUDA(ctx, cudaGetLastError());
     } else if (ctx->nc) {
-        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->max_deg,
+        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->classes,
                       ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, st);
         BM_CUDA(ctx, cudaGetLastError());
     }
@@ -1551,7 +1559,7 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     k_check_matching<<<grid_for(ctx, ctx->nr > ctx->nc ? ctx->nr : ctx->nc), ctx->block, 0, st>>>(ctx->nr, ctx->nc, ctx->rmatch, ctx->cmatch, ctx->ctl);
     BM_CUDA(ctx, cudaGetLastError());
     ctx->csr_ready = true;
-    ctx->max_deg = 0x7fffffff;  // (not read back)
+    ctx->classes = CLS_ALL;  // (not read back)
     if (ctx->opt.driver == BM_DRIVER_HOST) {
         rc = sync_ctl(ctx);
         if (rc) return rc;
@@ -1872,7 +1880,7 @@ int32_t bmi::enqueue_match(bmd::Params p, long long nnz, bool wr, int greedy, cu
     } else if (greedy) {
         // the cheap matching counts its lists in the control block's first two queue
         // counters, which the matching kernel needs at zero
-        launch_greedy(p.nr, p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, false, 0x7fffffff, rdeg, rdeg,
+        launch_greedy(p.nr, p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, false, CLS_ALL, rdeg, rdeg,
                       (int32_t*)p.queue, threads, B, st);
         if (cudaMemsetAsync(&p.ctl->qcnt[0], 0, 2 * sizeof(int32_t), st) != cudaSuccess) {
             (void)cudaGetLastError();

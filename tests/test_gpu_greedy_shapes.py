@@ -51,3 +51,12 @@ SHAPES = [(100000, 10, 5000), (40000, 300, 300), (33000, 1, 3000), (10, 40000, 3
 @pytest.mark.parametrize("block", [0, 64])
 def test_cheap_matching_of_few_columns_or_few_rows(shape, block):
     greedy(regular(*shape), block_size=block)
+
+
+@pytest.mark.parametrize("degrees", [[1], [2], [3], [8], [9, 32], [33], [2048], [2049], [2, 2049], [8, 33], [1, 9]], ids=str)
+def test_every_degree_class_by_itself_is_matched(degrees):
+    """Passes that no column needs are not launched; the others must be."""
+    rng = np.random.default_rng(degrees[0])
+    lists = [rng.choice(34000, degrees[c % len(degrees)], replace=False) for c in range(70)]
+    rm, cm = greedy(from_lists(34000, lists))  # more rows than the small graphs' kernel takes
+    assert np.all(cm >= 0)
