@@ -323,8 +323,60 @@ __device__ __forceinline__ int greedy_class(int d) {
     return d <= 2 ? CLS_2 : d <= 8 ? CLS_8 : d <= bmd::GREEDY_LIGHT ? CLS_LIGHT : d <= bmd::GREEDY_MEDIUM ? CLS_MEDIUM : CLS_HEAVY;
 }
 
-// rdeg (nullable, zero before): every row's number of entries, counted on the way for
-// the cheap matching.
+// Counts every row's entries in rdeg (zero before; nullptr: not counted) and returns whether a row id is out of
+// range.  A row's counter is one address, and additions to one address follow one another (0.7 ns each): a row
+// that all columns list, or few rows in all, held the count up far beyond the reading (1 M columns that share a
+// row: 0.65 ms of it; 3 M entries of 1,000 rows: 0.21 ms).  So a block keeps the counts of the first COUNT_SLOTS
+// rows it meets (by row id, one per slot) in shared memory and adds each to the row's counter once, at its end; only the
+// other rows' entries go to the counters one by one, and those rows are many and seldom the same.
+constexpr int COUNT_SLOTS = 4096;
+constexpr long long COUNT_DIRECT = 16384;  // entries of a graph up to which a counter cannot hold up for long
+__device__ __forceinline__ bool count_rows(int nr, long long nnz, const int32_t* __restrict__ ri, int32_t* rdeg) {
+    __shared__ int32_t s_row[COUNT_SLOTS], s_n[COUNT_SLOTS];
+    const bool slots = rdeg && nnz > COUNT_DIRECT;
+    if (slots) {
+        for (int i = threadIdx.x; i < COUNT_SLOTS; i += blockDim.x) {
+            s_row[i] = -1;
+            s_n[i] = 0;
+        }
+        __syncthreads();
+    }
+    const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long nthr = (long long)gridDim.x * blockDim.x;
+    bool bad = false;
+    for (long long e0 = tid; e0 < nnz; e0 += 4 * nthr) {
+        int r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) r[u] = e0 + u * nthr < nnz ? __ldg(&ri[e0 + u * nthr]) : 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (e0 + u * nthr >= nnz) continue;
+            if (r[u] < 0 || r[u] >= nr) {
+                bad = true;
+            } else if (slots) {
+                const int s = r[u] & (COUNT_SLOTS - 1);
+                int tag = *(volatile int32_t*)&s_row[s];
+                if (tag == -1) {
+                    tag = atomicCAS(&s_row[s], -1, r[u]);
+                    if (tag == -1) tag = r[u];
+                }
+                if (tag == r[u]) atomicAdd(&s_n[s], 1);
+                else atomicAdd(&rdeg[r[u]], 1);
+            } else if (rdeg) {
+                atomicAdd(&rdeg[r[u]], 1);
+            }
+        }
+    }
+    if (slots) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < COUNT_SLOTS; i += blockDim.x)
+            if (s_n[i]) atomicAdd(&rdeg[s_row[i]], s_n[i]);
+    }
+    return bad;
+}
+
+// COUNT: also counts the rows' entries in rdeg (count_rows).
+template <bool COUNT>
 __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __restrict__ cp,
                             const int32_t* __restrict__ ri, Ctl* ctl, int32_t* rdeg) {
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -339,12 +391,20 @@ __global__ void k_check_csr(int nr, int nc, long long nnz, const int32_t* __rest
     }
     classes = __reduce_or_sync(bmd::FULL, classes);
     if ((threadIdx.x & 31) == 0 && (classes & ~bmd::ld_volatile(&ctl->classes))) atomicOr(&ctl->classes, classes);
-    for (long long e = tid; e < nnz; e += nthr) {
-        int r = __ldg(&ri[e]);
-        if (r < 0 || r >= nr) bad = true;
-        else if (rdeg) atomicAdd(&rdeg[r], 1);
+    if (COUNT) {
+        bad |= count_rows(nr, nnz, ri, rdeg);
+    } else {
+        for (long long e = tid; e < nnz; e += nthr) {
+            const int r = __ldg(&ri[e]);
+            if (r < 0 || r >= nr) bad = true;
+        }
     }
     if (bad) bmd::set_error(ctl, BM_ERR_INVALID_CSR);
+}
+
+// The rows' entry counts of a CSR that has been checked.
+__global__ void k_count_rows(int nr, long long nnz, const int32_t* __restrict__ ri, int32_t* rdeg) {
+    count_rows(nr, nnz, ri, rdeg);
 }
 
 __global__ void k_check_matching(int nr, int nc, const int32_t* __restrict__ rm,
@@ -773,7 +833,8 @@ struct bm_ctx {
     int2* queue2 = nullptr;  // roots of the next phase (one-endpoint GPUBFS-WR)
     int32_t* endpoints = nullptr;
     int32_t* rvis = nullptr;     // per-row claim stamps of the persistent kernel
-    int32_t* rdeg = nullptr;     // per-row number of entries, counted by the CSR check (cheap matching)
+    int32_t* rdeg = nullptr;     // per-row number of entries, for the cheap matching (ensure_rdeg)
+    bool rdeg_ready = false;     // ... they are those of the present CSR
     int2* crec = nullptr;        // per-column (parent column, matched row) of the last search
     long long stamp_next = 0;    // every stamp in rvis is below stamp_next + 1
     int32_t* profile = nullptr;  // kProfileCap phases x 4
@@ -970,13 +1031,32 @@ bool starts_cheap(const bm_ctx* ctx) {
            ctx->opt.wr_one_endpoint == 1 && ctx->opt.driver == BM_DRIVER_PERSISTENT && !ctx->opt.deterministic;
 }
 
-int32_t validate_csr_async(bm_ctx* ctx) {
-    const long long work = ctx->nnz > ctx->nc ? ctx->nnz : (long long)ctx->nc + 1;
-    const int g = grid_for(ctx, (int)(work < (1 << 30) ? work : (1 << 30)));
-    if (ctx->nr) BM_CUDA(ctx, cudaMemsetAsync(ctx->rdeg, 0, 4 * (size_t)ctx->nr, ctx->stream));
-    k_check_csr<<<g, ctx->block, 0, ctx->stream>>>(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->ctl,
-                                                   ctx->rdeg);
+int edge_grid(bm_ctx* ctx) { return grid_for(ctx, (int)std::min(ctx->nnz > ctx->nc ? ctx->nnz : (int64_t)ctx->nc + 1, (int64_t)1 << 30)); }
+
+// Queues the CSR check; count: it counts the rows' entries too.
+int32_t validate_csr_async(bm_ctx* ctx, bool count) {
+    ctx->rdeg_ready = false;
+    if (count) {
+        if (ctx->nr) BM_CUDA(ctx, cudaMemsetAsync(ctx->rdeg, 0, 4 * (size_t)ctx->nr, ctx->stream));
+        k_check_csr<true><<<edge_grid(ctx), ctx->block, 0, ctx->stream>>>(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr,
+                                                                          ctx->row_idx, ctx->ctl, ctx->rdeg);
+    } else {
+        k_check_csr<false><<<edge_grid(ctx), ctx->block, 0, ctx->stream>>>(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr,
+                                                                           ctx->row_idx, ctx->ctl, nullptr);
+    }
     BM_CUDA(ctx, cudaGetLastError());
+    ctx->rdeg_ready = count;
+    return BM_OK;
+}
+
+// The rows' entry counts, which only the cheap matching of the default option reads: counted when it is first
+// called on a CSR (checked before), not with every CSR that arrives.
+int32_t ensure_rdeg(bm_ctx* ctx) {
+    if (ctx->rdeg_ready) return BM_OK;
+    if (ctx->nr) BM_CUDA(ctx, cudaMemsetAsync(ctx->rdeg, 0, 4 * (size_t)ctx->nr, ctx->stream));
+    if (ctx->nnz) k_count_rows<<<edge_grid(ctx), ctx->block, 0, ctx->stream>>>(ctx->nr, ctx->nnz, ctx->row_idx, ctx->rdeg);
+    BM_CUDA(ctx, cudaGetLastError());
+    ctx->rdeg_ready = true;
     return BM_OK;
 }
 
@@ -1109,6 +1189,8 @@ int32_t ensure_det_arena(bm_ctx* ctx) {
 int32_t run(bm_ctx* ctx, bool bfs_only) {
     Params p = make_params(ctx, bfs_only);
     if (!bfs_only && starts_cheap(ctx)) {
+        const int32_t rc = ensure_rdeg(ctx);
+        if (rc) return rc;
         // (its list counters are two of the queue counters, which the matching kernel needs at zero)
         launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, false,
                       ctx->classes, ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, ctx->stream);
@@ -1199,11 +1281,14 @@ bool solo_match(const bm_ctx* ctx) {
 }
 
 // The cheap matching on one block or cluster; |M| is in ctx->h_ctl when the stream has been waited for.
-cudaError_t run_solo_greedy(bm_ctx* ctx) {
+int32_t run_solo_greedy(bm_ctx* ctx) {
+    const int32_t rc = ensure_rdeg(ctx);
+    if (rc) return rc;
     const int C = solo_cluster(ctx);
     const size_t smem = 128 * ((((size_t)ctx->nr + 31) / 32 + C - 1) / C);
-    return launch_cluster(C == 1 ? bms1::k_solo_greedy<1, bms1::SOLO_T1> : bms1::k_solo_greedy<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream,
-                          make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl);
+    BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo_greedy<1, bms1::SOLO_T1> : bms1::k_solo_greedy<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream,
+                          make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl));
+    return BM_OK;
 }
 
 // The whole search on one block from (rm_src, cm_src); the outcome is in
@@ -1214,7 +1299,10 @@ int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool
     // (the cheap matching's kernel clears the control block, so not after input checks that report through it)
     const bool pre = !check_src && !check_err && starts_cheap(ctx);
     const bms1::SoloArgs a{rm_src, cm_src, rm_out, cm_out, ctx->h_ctl, check_src ? 1 : 0, check_err ? 1 : 0, pre ? 1 : 0};
-    if (pre) BM_CUDA(ctx, run_solo_greedy(ctx));
+    if (pre) {
+        const int32_t rc = run_solo_greedy(ctx);
+        if (rc) return rc;
+    }
     ctx->empty = false;
     const int C = solo_cluster(ctx);
     const size_t smem = bms1::Layout(ctx->nr, ctx->nc, ctx->nnz, C).bytes;
@@ -1368,7 +1456,7 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
         return BM_ERR_CUDA;
     }
     if (!own) {
-        rc = validate_csr_async(ctx);
+        rc = validate_csr_async(ctx, false);
         if (!rc) rc = sync_ctl(ctx);
         if (!rc && ctx->h_ctl->err) rc = ctx->h_ctl->err;
         if (rc) { bm_destroy(ctx); return rc; }
@@ -1400,7 +1488,7 @@ int32_t bm_upload_csr(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     BM_CUDA(ctx, cudaMemcpyAsync((void*)ctx->col_ptr, h_col_ptr, 4 * ((size_t)ctx->nc + 1), cudaMemcpyHostToDevice, st));
     if (ctx->nnz)
         BM_CUDA(ctx, cudaMemcpyAsync((void*)ctx->row_idx, h_row_idx, 4 * (size_t)ctx->nnz, cudaMemcpyHostToDevice, st));
-    int32_t rc = validate_csr_async(ctx);
+    int32_t rc = validate_csr_async(ctx, false);
     if (!rc) rc = sync_ctl(ctx);
     if (rc) return rc;
     if (ctx->h_ctl->err) { ctx->csr_ready = false; return ctx->h_ctl->err; }
@@ -1416,7 +1504,8 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
     cudaStream_t st = ctx->stream;
     ctx->empty = false;
     if (solo_cluster(ctx) > 0) {
-        BM_CUDA(ctx, run_solo_greedy(ctx));
+        const int32_t rc = run_solo_greedy(ctx);
+        if (rc) return rc;
         BM_CUDA(ctx, cudaStreamSynchronize(st));
         if (card_out) *card_out = ctx->h_ctl->card;
         return BM_OK;
@@ -1434,6 +1523,8 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
         BM_CUDA(ctx, cudaGetLastError());
     } else if (ctx->nc) {
+        const int32_t rc = ensure_rdeg(ctx);
+        if (rc) return rc;
         launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->classes,
                       ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, st);
         BM_CUDA(ctx, cudaGetLastError());
@@ -1554,7 +1645,8 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     }
     // input checks report through the control block; the match launch then
     // returns at once if one failed
-    int32_t rc = validate_csr_async(ctx);
+    const bool solo = solo_match(ctx);
+    int32_t rc = validate_csr_async(ctx, !solo && starts_cheap(ctx));
     if (rc) return rc;
     k_check_matching<<<grid_for(ctx, ctx->nr > ctx->nc ? ctx->nr : ctx->nc), ctx->block, 0, st>>>(ctx->nr, ctx->nc, ctx->rmatch, ctx->cmatch, ctx->ctl);
     BM_CUDA(ctx, cudaGetLastError());
@@ -1565,7 +1657,6 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
         if (rc) return rc;
         if (ctx->h_ctl->err) { ctx->csr_ready = false; return ctx->h_ctl->err; }
     }
-    const bool solo = solo_match(ctx);
     if (solo) {
         rc = run_solo(ctx, ctx->rmatch, ctx->cmatch, false, true, nullptr, nullptr, card_out, stats);
         if (rc < 0 && rc != BM_ERR_INVALID_CSR && rc != BM_ERR_INVALID_MATCHING) return rc;
@@ -1770,7 +1861,7 @@ extern "C" int32_t bm_match_noalloc(int32_t n_rows, int32_t n_cols, int64_t nnz,
     int g = (int)((work + d.block - 1) / d.block);
     if (g > threads) g = threads;
     if (g < 1) g = 1;
-    k_check_csr<<<g, d.block, 0, st>>>(n_rows, n_cols, nnz, col_ptr, row_idx, ctl, nullptr);
+    k_check_csr<false><<<g, d.block, 0, st>>>(n_rows, n_cols, nnz, col_ptr, row_idx, ctl, nullptr);
     const int n_max = n_rows > n_cols ? n_rows : n_cols;
     int g2 = (n_max + d.block - 1) / d.block;
     if (g2 > threads) g2 = threads;
@@ -1850,8 +1941,9 @@ int32_t bmi::enqueue_match(bmd::Params p, long long nnz, bool wr, int greedy, cu
     // the cheap matching's entry counts go where the search keeps its predecessors
     int32_t* const rdeg = greedy && !p.dkey ? p.pred : nullptr;
     if (rdeg && nr && cudaMemsetAsync(rdeg, 0, 4 * nr, st) != cudaSuccess) { (void)cudaGetLastError(); return BM_ERR_CUDA; }
-    k_check_csr<<<grid_of(nnz > p.nc ? nnz : (long long)p.nc + 1), B, 0, st>>>(p.nr, p.nc, nnz, p.col_ptr,
-                                                                               p.row_idx, p.ctl, rdeg);
+    const int eg = grid_of(nnz > p.nc ? nnz : (long long)p.nc + 1);
+    if (rdeg) k_check_csr<true><<<eg, B, 0, st>>>(p.nr, p.nc, nnz, p.col_ptr, p.row_idx, p.ctl, rdeg);
+    else k_check_csr<false><<<eg, B, 0, st>>>(p.nr, p.nc, nnz, p.col_ptr, p.row_idx, p.ctl, nullptr);
     if ((nr && (cudaMemsetAsync(p.rmatch, 0xff, 4 * nr, st) != cudaSuccess ||
                 cudaMemsetAsync(p.rvis, 0, 4 * nr, st) != cudaSuccess)) ||
         (nc && cudaMemsetAsync(p.cmatch, 0xff, 4 * nc, st) != cudaSuccess)) {

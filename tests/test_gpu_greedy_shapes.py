@@ -60,3 +60,51 @@ def test_every_degree_class_by_itself_is_matched(degrees):
     lists = [rng.choice(34000, degrees[c % len(degrees)], replace=False) for c in range(70)]
     rm, cm = greedy(from_lists(34000, lists))  # more rows than the small graphs' kernel takes
     assert np.all(cm >= 0)
+
+
+@pytest.mark.parametrize("first", [None, "deterministic", "host"])
+@pytest.mark.parametrize("n", [2000, 40000])  # small graphs' kernel / grid
+def test_counted_rows_decide_the_choice(n, first):
+    """Column c lists a row that all columns list, one that every 4,096th column lists too and one of its own, which
+    it must take, as the row of fewest entries.  The counts are made when the cheap matching first needs them, also
+    of a context whose CSR was checked under another option."""
+    # (no row has its column's number; the own rows' counting slots are those of the shared ones)
+    lists = [np.roll([n, n + 1 + c % 4096, n + 4097 + c], c % 3) for c in range(n)]
+    g = from_lists(2 * n + 4097, lists)
+
+    def deterministic(m):
+        m.greedy()
+        m.match()
+        m.set_options(deterministic=0)
+
+    def host(m):
+        m.set_options(driver=1)
+        m.match()
+        m.set_options(driver=0)
+
+    rm, cm = greedy(g, first={"deterministic": deterministic, "host": host}.get(first), deterministic=int(first == "deterministic"))
+    shared = np.bincount(1 + np.arange(n) % 4096, minlength=4097)[1 + np.arange(n) % 4096] > 1
+    assert np.array_equal(cm[shared], n + 4097 + np.flatnonzero(shared))
+
+
+def test_counts_follow_the_csr():
+    """A new CSR in the same context: its own counts, whichever call brought it."""
+    n = 40000
+    size = n + n // 2 + n  # rows: n that no column lists, n / 2 that two list, n that one lists
+    own = [np.array([n + n // 2 + c, n + c % (n // 2)]) for c in range(n)]
+    graphs = [from_lists(size, own), from_lists(size, [x[::-1].copy() for x in own])]
+    rm = torch.empty(size, dtype=torch.int32, device="cuda")
+    cm = torch.empty(n, dtype=torch.int32, device="cuda")
+    with bmatch.Matcher(size, n, 2 * n) as m:
+        for k, call in enumerate(["upload", "host", "host given", "upload", "host"]):
+            g = graphs[k % 2]
+            ri = n + (g.row_idx - n + 777 * k) % (size - n)  # every time another row numbering
+            if call == "upload":
+                m.upload_csr(g.col_ptr, ri)
+            else:
+                given = (np.full(size, -1, np.int32), np.full(n, -1, np.int32)) if call == "host given" else ()
+                assert m.match_host(g.col_ptr, ri, *given).card == n
+            m.set_matching()
+            assert m.greedy() == n
+            m.get_matching(rm, cm)
+            assert np.array_equal(cm.cpu().numpy(), n + (n // 2 + np.arange(n) + 777 * k) % (size - n))
