@@ -407,12 +407,14 @@ __device__ __forceinline__ void add_to_counter(long long* dst, unsigned v) {
 constexpr int GREEDY_LIGHT = 32;     // columns of at most this many rows: a thread each
 constexpr int GREEDY_MEDIUM = 2048;  // ... and this many: a warp each
 constexpr int GREEDY_U = 4;          // rows per thread and step of the cooperative scans
+constexpr int GREEDY_CROWD = 64;     // entries a row on average from which on columns crowd each other
 constexpr int GREEDY_TAKEN = -1;     // state of a matched row; a free row's is its number of entries
 
 // The free row with the fewest entries of a list of deg rows, the first such
 // from position rot on (wrapping); U rows per step with the loads in flight
-// together.  Returns the row (-1: none is free) and the state it was seen with.
-template <int U, class State>
+// together.  ANY: of the first step with a free row only.
+// Returns the row (-1: none is free) and the state it was seen with.
+template <int U, bool ANY, class State>
 __device__ __forceinline__ int greedy_pick(const int32_t* __restrict__ list, int deg, int rot, State state, int& seen) {
     int best_s = 0x7fffffff, best_r = -1;
     for (int i = 0; i < deg; i += U) {
@@ -427,17 +429,53 @@ __device__ __forceinline__ int greedy_pick(const int32_t* __restrict__ list, int
 #pragma unroll
         for (int u = 0; u < U; ++u)
             if (st[u] >= 0 && (st[u] < best_s || best_r < 0)) { best_s = st[u]; best_r = r[u]; }
+        if (ANY && best_r >= 0) break;
     }
     seen = best_s;
     return best_r;
 }
 
+// Rows of very many entries each: which of them a column takes matters little, and columns that list the same
+// ones get in each other's way.
+__host__ __device__ __forceinline__ bool greedy_crowded(int nr, long long nnz) { return nnz > (long long)GREEDY_CROWD * nr; }
+
+// A thread takes a free row of a list (greedy_pick); take(row, seen) claims it.  Columns that list the same rows
+// want the same one, and all but one lose.  A column that has lost twice takes the first free row that it finds
+// (each its own, from position rot on), not the next one that all the losers want; with any it does so at once
+// (crowded rows and more than twice as many columns).  100,000 columns of 30 of 1,000 rows, cheap matching: 565 us
+// when losers chose again, 394 us after two losses, 240 us with any.  After one loss already: 1 M columns of 10 of
+// 1 M rows end 4% further from the maximum and take a phase more (902 -> 1,040 us with the search).
+template <int U, class State, class Take>
+__device__ __forceinline__ int greedy_thread(const int32_t* __restrict__ list, int deg, int rot, bool any, State state,
+                                             Take take) {
+    int seen;
+    if (!any) {
+#pragma unroll 1
+        for (int tries = 0; tries < 2; ++tries) {
+            const int r = greedy_pick<U, false>(list, deg, rot, state, seen);
+            if (r < 0 || take(r, seen)) return r;
+        }
+    }
+    for (;;) {
+        const int r = greedy_pick<U, true>(list, deg, rot, state, seen);
+        if (r < 0 || take(r, seen)) return r;
+    }
+}
+
 // A warp takes a free row of a list of n rows: 32 x GREEDY_U rows per step, of
-// the first step with a free row the one with the fewest entries that no one
-// takes meanwhile.  Returns the row (every lane; -1: none).
+// the first step with a free row the one that greedy_pick would take; if that is
+// lost, or with any (crowded rows), the first free
+// one from lane `spread` on.  Returns the row (every lane; -1: none).  After a
+// loss the step's rows are looked at again: columns that share most rows (30
+// dense blocks of 300 x 300, all at work at once) otherwise tried every row of
+// it that others had taken (315 -> 64 us; 2,000 columns of 1,000 of 2,000 rows
+// 140 -> 51 us, 40,000 of 100 of 40,000 135 -> 75 us).
 template <class State, class Take>
-__device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int n, State state_of, Take take) {
+__device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int n, unsigned spread, bool any, State state_of,
+                                           Take take) {
     const int lane = threadIdx.x & 31;
+    bool first = true;
+    spread &= 31;
     for (int e0 = 0; e0 < n; e0 += 32 * GREEDY_U) {  // warp-uniform
         int r[GREEDY_U], st[GREEDY_U];
 #pragma unroll
@@ -447,23 +485,26 @@ __device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int
         }
 #pragma unroll
         for (int u = 0; u < GREEDY_U; ++u) st[u] = r[u] >= 0 ? state_of(r[u]) : GREEDY_TAKEN;
-        for (;;) {  // warp-uniform: the window's free row with the fewest entries
+        for (;;) {  // warp-uniform
             int best_s = 0x7fffffff, best_u = -1, best_r = -1;
 #pragma unroll
             for (int u = 0; u < GREEDY_U; ++u)
-                if (st[u] >= 0 && (st[u] < best_s || best_u < 0)) { best_s = st[u]; best_u = u; best_r = r[u]; }
-            if (!__any_sync(FULL, best_u >= 0)) break;  // none left: the next window
-            const int least = __reduce_min_sync(FULL, best_u >= 0 ? best_s : 0x7fffffff);
-            const int l = __ffs(__ballot_sync(FULL, best_u >= 0 && best_s == least)) - 1;
-            int won = -1;
-            if (lane == l) {
-                if (take(best_r, best_s)) won = best_r;
-#pragma unroll
-                for (int u = 0; u < GREEDY_U; ++u)
-                    if (u == best_u) st[u] = GREEDY_TAKEN;
+                if (st[u] >= 0 && (best_u < 0 || (!any && st[u] < best_s))) { best_s = st[u]; best_u = u; best_r = r[u]; }
+            const unsigned free_lanes = __ballot_sync(FULL, best_u >= 0);
+            if (!free_lanes) break;  // none left: the next window
+            int l = (__ffs(__funnelshift_r(free_lanes, free_lanes, spread)) - 1 + (int)spread) & 31;
+            if (first && !any) {
+                const int least = __reduce_min_sync(FULL, best_u >= 0 ? best_s : 0x7fffffff);
+                l = __ffs(__ballot_sync(FULL, best_u >= 0 && best_s == least)) - 1;
             }
+            int won = -1;
+            if (lane == l && take(best_r, best_s)) won = best_r;
             won = __shfl_sync(FULL, won, l);
             if (won >= 0) return won;
+            // lost: others have taken rows of this window meanwhile, so look again (the row lost reads as taken)
+            first = false;
+#pragma unroll
+            for (int u = 0; u < GREEDY_U; ++u) st[u] = st[u] >= 0 ? state_of(r[u]) : GREEDY_TAKEN;
         }
     }
     return -1;

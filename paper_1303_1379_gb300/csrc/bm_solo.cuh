@@ -695,6 +695,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     auto state_of = [&](int r) { return (int)dld32(state_at(r)); };
     auto take = [&](int r, int seen) { return dcas(state_at(r), seen, GREEDY_TAKEN) == seen; };
     const int limit[4] = {0, 2, 8, GREEDY_LIGHT};
+    const bool crowded = greedy_crowded(nr, __ldg(&p.col_ptr[nc])), any = crowded && nc > 2LL * nr;
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
         for (unsigned k0 = warp; k0 < (1u << bits); k0 += T / 32) {
@@ -706,16 +707,11 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
             if (k == 0 && deg > GREEDY_LIGHT) longs[atomicAdd(&s_long, 1)] = c;
             if (deg <= limit[k] || deg > limit[k + 1] || p.cmatch[c] != -1) continue;
             const int rot = (int)__umulhi(hash32((unsigned)c), (unsigned)deg);
-            for (;;) {
-                int seen;
-                const int r = greedy_pick<4>(p.row_idx + beg, deg, rot, state_of, seen);
-                if (r < 0) break;  // every row is taken
-                if (take(r, seen)) {
-                    p.rmatch[r] = c;
-                    p.cmatch[c] = r;
-                    ++n;
-                    break;
-                }
+            const int r = greedy_thread<4>(p.row_idx + beg, deg, rot, any, state_of, take);
+            if (r >= 0) {
+                p.rmatch[r] = c;
+                p.cmatch[c] = r;
+                ++n;
             }
         }
         cluster_sync<C>();
@@ -723,8 +719,8 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     for (int k = warp; k < s_long; k += T / 32) {  // warp-uniform
         const int c = longs[k];
         if (p.cmatch[c] != -1) continue;
-        const int beg = __ldg(&p.col_ptr[c]);
-        const int r = greedy_warp(p.row_idx + beg, __ldg(&p.col_ptr[c + 1]) - beg, state_of, take);
+        const int beg = __ldg(&p.col_ptr[c]), deg = __ldg(&p.col_ptr[c + 1]) - beg;
+        const int r = greedy_warp(p.row_idx + beg, deg, hash32((unsigned)c), crowded, state_of, take);
         if (r >= 0 && lane == 0) {
             p.rmatch[r] = c;
             p.cmatch[c] = r;

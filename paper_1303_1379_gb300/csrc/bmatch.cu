@@ -531,7 +531,7 @@ __global__ void k_greedy_state(int nr, const int32_t* __restrict__ rm, const int
 // Columns of LO < degree <= HI; LISTS: also lists the columns of the later passes.
 template <int LO, int HI, bool LISTS>
 __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int32_t* __restrict__ ri,
-                               int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl, Ctl* ctl) {
+                               int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl, Ctl* ctl, bool any) {
     // after an asynchronous CSR check on the same stream: an invalid CSR is not read
     if (bmd::ld_volatile(&ctl->err) != 0) return;
     int n = 0;  // columns this thread matched (LISTS: and those that were)
@@ -558,23 +558,20 @@ __global__ void k_greedy_light(int nc, const int32_t* __restrict__ cp, const int
             if (deg > HI) continue;
         }
         const int rot = (int)__umulhi(bmd::hash32((unsigned)c), (unsigned)deg);
-        for (;;) {
-            int seen;
-            const int r = bmd::greedy_pick<U>(ri + beg, deg, rot, [&](int k) { return bmd::ld_volatile(&state[k]); }, seen);
-            if (r < 0) break;  // every row is taken
-            if (atomicCAS(&state[r], seen, GREEDY_TAKEN) == seen) {
-                rm[r] = c;
-                cm[c] = r;
-                ++n;
-                break;
-            }
+        const int r = bmd::greedy_thread<U>(
+            ri + beg, deg, rot, any, [&](int k) { return bmd::ld_volatile(&state[k]); },
+            [&](int k, int seen) { return atomicCAS(&state[k], seen, GREEDY_TAKEN) == seen; });
+        if (r >= 0) {
+            rm[r] = c;
+            cm[c] = r;
+            ++n;
         }
     }
     block_count(&ctl->card, n);
 }
 
-__global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri, int32_t* state,
-                                int32_t* rm, int32_t* cm, GreedyLists gl, Ctl* ctl) {
+__global__ void __launch_bounds__(1024, 2) k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* __restrict__ ri, int32_t* state,
+                                int32_t* rm, int32_t* cm, GreedyLists gl, Ctl* ctl, bool any) {
     if (bmd::ld_volatile(&ctl->err) != 0) return;
     int won = 0;
     const int lane = threadIdx.x & 31;
@@ -585,7 +582,7 @@ __global__ void k_greedy_medium(const int32_t* __restrict__ cp, const int32_t* _
         const int hc = gl.medium[k];
         const int hb = __ldg(&cp[hc]), he = __ldg(&cp[hc + 1]);
         const int r = bmd::greedy_warp(
-            ri + hb, he - hb, [&](int k) { return bmd::ld_volatile(&state[k]); },
+            ri + hb, he - hb, bmd::hash32((unsigned)hc), any, [&](int k) { return bmd::ld_volatile(&state[k]); },
             [&](int k, int seen) { return atomicCAS(&state[k], seen, GREEDY_TAKEN) == seen; });
         if (r >= 0 && lane == 0) {
             rm[r] = hc;
@@ -675,17 +672,19 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
 // once).  All sized by the columns, few columns and many rows or long lists
 // ran on a block or two (10 columns of 5,000 of 100,000 rows 135 -> 36 us, 1,000
 // columns of 300 of 100,000 rows 127 -> 37 us).
-void launch_greedy(int nr, int nc, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, Ctl* ctl, bool clear,
+void launch_greedy(int nr, int nc, long long nnz, const int32_t* cp, const int32_t* ri, int32_t* rm, int32_t* cm, Ctl* ctl, bool clear,
                    int classes, const int32_t* rdeg, int32_t* state, int32_t* lists, int cap, int block,
                    cudaStream_t st) {
     const GreedyLists gl{lists, lists + nc, &ctl->qcnt[0]};
     auto blocks = [&](long long threads) { return (int)std::max(1LL, std::min((threads + block - 1) / block, (long long)cap)); };
     const int grid = blocks(nc);
+    const bool crowded = bmd::greedy_crowded(nr, nnz);
+    const bool any = crowded && nc > 2LL * nr;
     k_greedy_state<<<blocks(nr), block, 0, st>>>(nr, rm, rdeg, state, clear ? ctl : nullptr);
-    k_greedy_light<0, 2, true><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    if (classes & CLS_8) k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    if (classes & CLS_LIGHT) k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl);
-    if (classes & CLS_MEDIUM) k_greedy_medium<<<blocks(32LL * nc), block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
+    k_greedy_light<0, 2, true><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl, any);
+    if (classes & CLS_8) k_greedy_light<2, 8, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl, any);
+    if (classes & CLS_LIGHT) k_greedy_light<8, GREEDY_LIGHT, false><<<grid, block, 0, st>>>(nc, cp, ri, state, rm, cm, gl, ctl, any);
+    if (classes & CLS_MEDIUM) k_greedy_medium<<<blocks(32LL * nc), block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl, crowded);
     if (classes & CLS_HEAVY)
         k_greedy_heavy<<<blocks((long long)block * nc), block, 0, st>>>(cp, ri, state, rm, cm, gl, ctl);
 }
@@ -1192,7 +1191,7 @@ int32_t run(bm_ctx* ctx, bool bfs_only) {
         const int32_t rc = ensure_rdeg(ctx);
         if (rc) return rc;
         // (its list counters are two of the queue counters, which the matching kernel needs at zero)
-        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, false,
+        launch_greedy(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, false,
                       ctx->classes, ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, ctx->stream);
         BM_CUDA(ctx, cudaGetLastError());
         BM_CUDA(ctx, cudaMemsetAsync(&ctx->ctl->qcnt[0], 0, 2 * sizeof(int32_t), ctx->stream));
@@ -1525,7 +1524,7 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
     } else if (ctx->nc) {
         const int32_t rc = ensure_rdeg(ctx);
         if (rc) return rc;
-        launch_greedy(ctx->nr, ctx->nc, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->classes,
+        launch_greedy(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->classes,
                       ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, st);
         BM_CUDA(ctx, cudaGetLastError());
     }
@@ -1972,7 +1971,7 @@ int32_t bmi::enqueue_match(bmd::Params p, long long nnz, bool wr, int greedy, cu
     } else if (greedy) {
         // the cheap matching counts its lists in the control block's first two queue
         // counters, which the matching kernel needs at zero
-        launch_greedy(p.nr, p.nc, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, false, CLS_ALL, rdeg, rdeg,
+        launch_greedy(p.nr, p.nc, nnz, p.col_ptr, p.row_idx, p.rmatch, p.cmatch, p.ctl, false, CLS_ALL, rdeg, rdeg,
                       (int32_t*)p.queue, threads, B, st);
         if (cudaMemsetAsync(&p.ctl->qcnt[0], 0, 2 * sizeof(int32_t), st) != cudaSuccess) {
             (void)cudaGetLastError();

@@ -108,3 +108,11 @@ def test_counts_follow_the_csr():
             assert m.greedy() == n
             m.get_matching(rm, cm)
             assert np.array_equal(cm.cpu().numpy(), n + (n // 2 + np.arange(n) + 777 * k) % (size - n))
+
+
+@pytest.mark.parametrize("n,k,cols", [(40, 30, 30), (100, 300, 300), (2, 1200, 400), (2, 2500, 400)])
+def test_columns_that_list_the_same_rows(n, k, cols):
+    """n blocks of columns that all list the same k rows: every one of them gets one."""
+    lists = [b * k + np.roll(np.arange(k), 7 * c) for b in range(n) for c in range(cols)]
+    rm, cm = greedy(from_lists(34000, lists))
+    assert np.all(cm >= 0)
