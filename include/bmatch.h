@@ -179,8 +179,10 @@ BM_API int32_t bm_set_options(bm_ctx *ctx, const bm_options *opt);
 
 /* Cheap initial matching on the GPU (the "cheap matching" initialisation of
  * Section 4): every unmatched column claims, with an atomic compare-and-swap,
- * the unmatched row of its list that the fewest columns list (ties: from a
- * position of the list that depends on the column id).  Columns are taken by
+ * the unmatched row of its list that has its own number, else the one that the
+ * fewest columns list (ties: from a position of the list that depends on the
+ * column id); a column that loses the row it wants twice, or one of a graph
+ * with more than 64 entries a row, any unmatched one.  Columns are taken by
  * degree, shortest lists first (up to 2, 8 and 32 rows: a thread each and the
  * whole list; up to 2048: a warp each, longer: a block each, both dealt from
  * lists the first pass builds in the context's queue and scanned up to the

@@ -410,13 +410,15 @@ constexpr int GREEDY_U = 4;          // rows per thread and step of the cooperat
 constexpr int GREEDY_CROWD = 64;     // entries a row on average from which on columns crowd each other
 constexpr int GREEDY_TAKEN = -1;     // state of a matched row; a free row's is its number of entries
 
-// The free row with the fewest entries of a list of deg rows, the first such
-// from position rot on (wrapping); U rows per step with the loads in flight
-// together.  ANY: of the first step with a free row only.
+// The free row of a list of deg rows that a column takes: the one with the
+// column's own number (diag) if that is listed, else the one with the fewest
+// entries, the first such from position rot on (wrapping); U rows per step with
+// the loads in flight together.  ANY: of the first step with a free row only.
 // Returns the row (-1: none is free) and the state it was seen with.
 template <int U, bool ANY, class State>
-__device__ __forceinline__ int greedy_pick(const int32_t* __restrict__ list, int deg, int rot, State state, int& seen) {
-    int best_s = 0x7fffffff, best_r = -1;
+__device__ __forceinline__ int greedy_pick(const int32_t* __restrict__ list, int deg, int rot, int diag, State state,
+                                           int& seen) {
+    int best_s = 0x7fffffff, best_k = 0x7fffffff, best_r = -1;
     for (int i = 0; i < deg; i += U) {
         int r[U], st[U];
 #pragma unroll
@@ -427,8 +429,10 @@ __device__ __forceinline__ int greedy_pick(const int32_t* __restrict__ list, int
 #pragma unroll
         for (int u = 0; u < U; ++u) st[u] = r[u] >= 0 ? state(r[u]) : GREEDY_TAKEN;
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (st[u] >= 0 && (st[u] < best_s || best_r < 0)) { best_s = st[u]; best_r = r[u]; }
+        for (int u = 0; u < U; ++u) {
+            const int k = r[u] == diag ? -1 : st[u];
+            if (st[u] >= 0 && (k < best_k || best_r < 0)) { best_k = k; best_s = st[u]; best_r = r[u]; }
+        }
         if (ANY && best_r >= 0) break;
     }
     seen = best_s;
@@ -446,33 +450,33 @@ __host__ __device__ __forceinline__ bool greedy_crowded(int nr, long long nnz) {
 // when losers chose again, 394 us after two losses, 240 us with any.  After one loss already: 1 M columns of 10 of
 // 1 M rows end 4% further from the maximum and take a phase more (902 -> 1,040 us with the search).
 template <int U, class State, class Take>
-__device__ __forceinline__ int greedy_thread(const int32_t* __restrict__ list, int deg, int rot, bool any, State state,
-                                             Take take) {
+__device__ __forceinline__ int greedy_thread(const int32_t* __restrict__ list, int deg, int rot, int diag, bool any,
+                                             State state, Take take) {
     int seen;
     if (!any) {
 #pragma unroll 1
         for (int tries = 0; tries < 2; ++tries) {
-            const int r = greedy_pick<U, false>(list, deg, rot, state, seen);
+            const int r = greedy_pick<U, false>(list, deg, rot, diag, state, seen);
             if (r < 0 || take(r, seen)) return r;
         }
     }
     for (;;) {
-        const int r = greedy_pick<U, true>(list, deg, rot, state, seen);
+        const int r = greedy_pick<U, true>(list, deg, rot, diag, state, seen);
         if (r < 0 || take(r, seen)) return r;
     }
 }
 
 // A warp takes a free row of a list of n rows: 32 x GREEDY_U rows per step, of
 // the first step with a free row the one that greedy_pick would take; if that is
-// lost, or with any (crowded rows), the first free
+// lost, or with any (crowded rows: only the own number first), the first free
 // one from lane `spread` on.  Returns the row (every lane; -1: none).  After a
 // loss the step's rows are looked at again: columns that share most rows (30
 // dense blocks of 300 x 300, all at work at once) otherwise tried every row of
 // it that others had taken (315 -> 64 us; 2,000 columns of 1,000 of 2,000 rows
 // 140 -> 51 us, 40,000 of 100 of 40,000 135 -> 75 us).
 template <class State, class Take>
-__device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int n, unsigned spread, bool any, State state_of,
-                                           Take take) {
+__device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int n, int diag, unsigned spread, bool any,
+                                           State state_of, Take take) {
     const int lane = threadIdx.x & 31;
     bool first = true;
     spread &= 31;
@@ -493,9 +497,21 @@ __device__ __forceinline__ int greedy_warp(const int32_t* __restrict__ list, int
             const unsigned free_lanes = __ballot_sync(FULL, best_u >= 0);
             if (!free_lanes) break;  // none left: the next window
             int l = (__ffs(__funnelshift_r(free_lanes, free_lanes, spread)) - 1 + (int)spread) & 31;
-            if (first && !any) {
-                const int least = __reduce_min_sync(FULL, best_u >= 0 ? best_s : 0x7fffffff);
-                l = __ffs(__ballot_sync(FULL, best_u >= 0 && best_s == least)) - 1;
+            if (first) {
+                int own = -1;
+#pragma unroll
+                for (int u = 0; u < GREEDY_U; ++u)
+                    if (r[u] == diag && st[u] >= 0) own = u;
+                const unsigned has = __ballot_sync(FULL, own >= 0);
+                if (has) {
+                    l = __ffs(has) - 1;
+#pragma unroll
+                    for (int u = 0; u < GREEDY_U; ++u)
+                        if (u == own) { best_u = u; best_r = r[u]; best_s = st[u]; }
+                } else if (!any) {
+                    const int least = __reduce_min_sync(FULL, best_u >= 0 ? best_s : 0x7fffffff);
+                    l = __ffs(__ballot_sync(FULL, best_u >= 0 && best_s == least)) - 1;
+                }
             }
             int won = -1;
             if (lane == l && take(best_r, best_s)) won = best_r;
@@ -1590,7 +1606,8 @@ __device__ __forceinline__ void block_greedy_sb(const Params& p) {
 #pragma unroll
             for (int v = 0; v < GU; ++v)
 #pragma unroll
-                for (int u = 0; u < GW; ++u) d[v][u] = r[v][u] >= 0 && !sb_test(p.vis, r[v][u]) ? p.rdeg8[r[v][u]] : 256;
+                for (int u = 0; u < GW; ++u)
+                    d[v][u] = r[v][u] < 0 || sb_test(p.vis, r[v][u]) ? 256 : r[v][u] == c[v] ? 0 : p.rdeg8[r[v][u]];
             bool more = false;
 #pragma unroll
             for (int v = 0; v < GU; ++v) {

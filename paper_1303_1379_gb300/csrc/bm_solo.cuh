@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
             if (k == 0 && deg > GREEDY_LIGHT) longs[atomicAdd(&s_long, 1)] = c;
             if (deg <= limit[k] || deg > limit[k + 1] || p.cmatch[c] != -1) continue;
             const int rot = (int)__umulhi(hash32((unsigned)c), (unsigned)deg);
-            const int r = greedy_thread<4>(p.row_idx + beg, deg, rot, any, state_of, take);
+            const int r = greedy_thread<4>(p.row_idx + beg, deg, rot, c, any, state_of, take);
             if (r >= 0) {
                 p.rmatch[r] = c;
                 p.cmatch[c] = r;
@@ -720,7 +720,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
         const int c = longs[k];
         if (p.cmatch[c] != -1) continue;
         const int beg = __ldg(&p.col_ptr[c]), deg = __ldg(&p.col_ptr[c + 1]) - beg;
-        const int r = greedy_warp(p.row_idx + beg, deg, hash32((unsigned)c), crowded, state_of, take);
+        const int r = greedy_warp(p.row_idx + beg, deg, c, hash32((unsigned)c), crowded, state_of, take);
         if (r >= 0 && lane == 0) {
             p.rmatch[r] = c;
             p.cmatch[c] = r;

@@ -116,3 +116,34 @@ def test_columns_that_list_the_same_rows(n, k, cols):
     lists = [b * k + np.roll(np.arange(k), 7 * c) for b in range(n) for c in range(cols)]
     rm, cm = greedy(from_lists(34000, lists))
     assert np.all(cm >= 0)
+
+
+def banded(n, offsets):
+    rows = np.arange(n)[:, None] + np.array(offsets)[None, :]
+    ok = (rows >= 0) & (rows < n)
+    return synth.Graph(n, n, np.concatenate([[0], np.cumsum(ok.sum(1))]).astype(np.int32), rows[ok].astype(np.int32), "banded")
+
+
+@pytest.mark.parametrize("n", [1000, 20000, 40000])  # one block, cluster, grid
+@pytest.mark.parametrize("offsets", [(0, 1), (-1, 0), (-1, 0, 1), tuple(range(-20, 21)), tuple(range(0, 1200))], ids=len)
+def test_a_whole_diagonal_is_taken(n, offsets):
+    """Bidiagonal matrices have one maximum matching, which no other choice than the diagonal finds."""
+    g = banded(n, offsets if len(offsets) < 100 or n > 2000 else offsets[:700])
+    if g.nnz > 30_000_000:
+        g = banded(n, offsets[:100])
+    rm, cm = greedy(g)
+    assert np.array_equal(cm, np.arange(n))
+
+
+def test_a_batch_takes_the_diagonal():
+    graphs = [banded(n, o) for n in (50, 3000) for o in ((0, 1), (-1, 0), (-3, -2, -1, 0, 1, 2, 3))]
+    off = [np.concatenate([[0], np.cumsum([f(g) for g in graphs])]).astype(np.int64)
+           for f in (lambda g: g.n_rows, lambda g: g.n_cols, lambda g: g.nnz)]
+    b = synth.Batch(np.array([g.n_rows for g in graphs], np.int32), np.array([g.n_cols for g in graphs], np.int32), *off,
+                    np.concatenate([g.col_ptr for g in graphs]), np.concatenate([g.row_idx for g in graphs]))
+    with bmatch.Batch.from_synth(b) as bb:
+        rm = torch.full((int(off[0][-1]),), -1, dtype=torch.int32, device="cuda")
+        cm = torch.full((int(off[1][-1]),), -1, dtype=torch.int32, device="cuda")
+        bb.match(rm, cm)
+    for k, g in enumerate(graphs):
+        assert np.array_equal(cm[off[1][k]:off[1][k + 1]].cpu().numpy(), np.arange(g.n_cols))
