@@ -497,11 +497,15 @@ __global__ void k_fill(int32_t* a, long long n, int v) {
 //    per step).  The first launch lists the last two kinds (R-MAT puts its
 //    hubs at neighbouring ids, so those passes deal them out from these lists
 //    instead of by id); their scans stop at the first step with a free row.
+//    The long ones choose by the same rule: a hub matched to a row that only
+//    hubs list is seldom reached by the search, one matched to the first free
+//    row is and then has its whole list read (R-MAT scale 21: search 640 ->
+//    550 us; 200,000 columns of 3 with 50 of 20,000 rows 855 -> 290 us).
 // state[r] is the row's number of entries while it is free and GREEDY_TAKEN
 // once it is matched, so one gather per entry answers both questions; the CAS
 // is on it, and its winner stores the two matches (no launch reads another
 // column's).  R-MAT scale 21: 284 us (first free row in list order: 262 us),
-// start 578.8 k of 587.2 k pairs (530.1 k), the search 640 us (without trees
+// start 578.8 k of 587.2 k pairs (530.1 k), the search 550 us (without trees
 // carried over 800 us; from the first free rows 1,042 us).
 using bmd::GREEDY_LIGHT;
 using bmd::GREEDY_MEDIUM;
@@ -603,7 +607,8 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
                                                        int32_t* state, int32_t* rm, int32_t* cm, GreedyLists gl,
                                                        Ctl* ctl) {
     if (bmd::ld_volatile(&ctl->err) != 0) return;
-    __shared__ int s_pos, s_done;
+    __shared__ unsigned long long s_best;
+    __shared__ int s_done;
     const int T = blockDim.x, t = threadIdx.x;
     const int n = gl.count[1];
     for (int k = blockIdx.x; k < n; k += gridDim.x) {  // block-uniform
@@ -611,7 +616,7 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
         const int hb = __ldg(&cp[hc]), he = __ldg(&cp[hc + 1]);
         if (t == 0) s_done = 0;
         __syncthreads();
-        for (int e0 = hb; e0 < he; e0 += T * GREEDY_U) {  // block-uniform
+        for (int e0 = hb; e0 < he && !s_done; e0 += T * GREEDY_U) {  // block-uniform
             int r[GREEDY_U], m[GREEDY_U];
 #pragma unroll
             for (int u = 0; u < GREEDY_U; ++u) {
@@ -620,44 +625,39 @@ __global__ void __launch_bounds__(1024) k_greedy_heavy(const int32_t* __restrict
             }
 #pragma unroll
             for (int u = 0; u < GREEDY_U; ++u) m[u] = r[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
-            // window position of this thread's first free row (list order: u major, thread minor)
-            int pos = 0x7fffffff;
+            for (;;) {  // block-uniform: the window's free row that greedy_pick would take, until one is won
+                int best_k = 0x7fffffff, best_u = 0;
 #pragma unroll
-            for (int u = GREEDY_U - 1; u >= 0; --u)
-                if (m[u] >= 0) pos = u * T + t;
-            if (t == 0) s_pos = 0x7fffffff;
-            __syncthreads();
-            if (pos != 0x7fffffff) atomicMin(&s_pos, pos);
-            __syncthreads();
-            // candidates in list order; a failed CAS (taken meanwhile) moves on to the next free one
-            while (s_pos != 0x7fffffff && !s_done) {  // block-uniform
-                const int mypos = s_pos;
-                __syncthreads();  // every thread has read s_pos
-                if (t == mypos % T) {
-                    const int u = mypos / T;
+                for (int u = 0; u < GREEDY_U; ++u) {
+                    const int key = r[u] == hc ? -1 : m[u];
+                    if (m[u] >= 0 && key < best_k) { best_k = key; best_u = u; }
+                }
+                if (t == 0) s_best = ~0ull;
+                __syncthreads();
+                if (best_k != 0x7fffffff)
+                    atomicMin(&s_best, (unsigned long long)(unsigned)(best_k + 1) << 32 | (unsigned)(best_u * T + t));
+                __syncthreads();
+                const unsigned long long best = s_best;
+                if (best == ~0ull) break;  // none left: the next window
+                const int pos = (int)(unsigned)(best & 0xffffffffull);
+                if (pos % T == t) {
                     int rr = -1, seen = 0;
 #pragma unroll
-                    for (int v = 0; v < GREEDY_U; ++v)
-                        if (v == u) { rr = r[v]; seen = m[v]; }
+                    for (int u = 0; u < GREEDY_U; ++u)
+                        if (u == pos / T) { rr = r[u]; seen = m[u]; }
                     if (atomicCAS(&state[rr], seen, GREEDY_TAKEN) == seen) {
                         rm[rr] = hc;
                         cm[hc] = rr;
                         atomicAdd(&ctl->card, 1);
                         s_done = 1;
                     }
-                    s_pos = 0x7fffffff;
                 }
                 __syncthreads();
-                if (!s_done) {
-                    int next = 0x7fffffff;
+                if (s_done) break;
+                // lost: others have taken rows of this window meanwhile (the one lost reads as taken)
 #pragma unroll
-                    for (int u = GREEDY_U - 1; u >= 0; --u)
-                        if (m[u] >= 0 && u * T + t > mypos) next = u * T + t;
-                    if (next != 0x7fffffff) atomicMin(&s_pos, next);
-                }
-                __syncthreads();
+                for (int u = 0; u < GREEDY_U; ++u) m[u] = m[u] >= 0 ? bmd::ld_volatile(&state[r[u]]) : GREEDY_TAKEN;
             }
-            if (s_done) break;
         }
         __syncthreads();  // s_done is reset for the next column
     }

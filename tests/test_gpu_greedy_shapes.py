@@ -147,3 +147,12 @@ def test_a_batch_takes_the_diagonal():
         bb.match(rm, cm)
     for k, g in enumerate(graphs):
         assert np.array_equal(cm[off[1][k]:off[1][k + 1]].cpu().numpy(), np.arange(g.n_cols))
+
+
+@pytest.mark.parametrize("block", [0, 1024])
+def test_hub_columns_take_the_row_of_fewest_entries(block):
+    """Eight columns of 3,000 rows, all but one of them shared: the one, in the middle of the first step's rows."""
+    lists = [100 + np.concatenate([np.arange(1000), [2999 + h], np.arange(1000, 2999)]) for h in range(8)]
+    lists += [np.array([5000 + c]) for c in range(33000)]
+    rm, cm = greedy(from_lists(40000, lists), block_size=block)
+    assert np.array_equal(cm[:8], 100 + 2999 + np.arange(8))
