@@ -156,3 +156,16 @@ def test_hub_columns_take_the_row_of_fewest_entries(block):
     lists += [np.array([5000 + c]) for c in range(33000)]
     rm, cm = greedy(from_lists(40000, lists), block_size=block)
     assert np.array_equal(cm[:8], 100 + 2999 + np.arange(8))
+
+
+@pytest.mark.parametrize("shape", [(600, 40000, 30), (1500, 40000, 3), (34000, 34000, 3)], ids=str)
+def test_first_phase_from_nothing(shape):
+    """One level, whether the cheap matching's kernels run it or (many more columns than rows) the search."""
+    g = regular(*shape)
+    cp, ri = to_dev(g)
+    with bmatch.Matcher(g.n_rows, g.n_cols, g.nnz, cp, ri) as m:
+        res = m.match()
+        levels, ends, _, _ = m.phase_profile()
+    want = oracle_max(g)
+    assert res.card == want == ends.sum() == res.stats["endpoints"] and res.stats["initial_card"] == 0
+    assert ends[0] > 0.5 * want and levels.sum() == res.stats["levels"]
