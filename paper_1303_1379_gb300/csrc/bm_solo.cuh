@@ -56,6 +56,7 @@ constexpr int SOLO_MAX = 0xfffe;       // rows and columns with a 16-bit id
 constexpr int SOLO_SMEM = 216 * 1024;  // dynamic shared memory of a block
 constexpr int PART = 128;              // a listed column's rows are expanded in parts of this many
 constexpr int SOLO_U = 2;              // edges of a thread in flight
+constexpr int SOLO_PASS = 2;           // status: the search is left to the grid
 constexpr int ROW_GLOBAL = 1 << 30;    // marks row positions in the graph's own row_idx
 
 struct SoloArgs {
@@ -67,6 +68,7 @@ struct SoloArgs {
     int32_t check_src;      // check that rm_src / cm_src are in range and inverse to each other
     int32_t check_err;      // p.ctl holds the outcome of input checks queued before
     int32_t pre;            // the first phase was run as a cheap matching, from the empty matching
+    int32_t max_roots;      // from more roots than this nothing is done, and the status is SOLO_PASS
 };
 
 // Where a block keeps what, in bytes from its dynamic shared memory's start.
@@ -371,7 +373,7 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
     end_step(true);
     int n_roots = sum_cnt, n_free = sum_eps, n_front = sum_cnt;
     int initial = nc - n_free;
-    int status = flag, phases = 0, no_roots = 0;
+    int status = flag == 0 && n_roots > a.max_roots ? SOLO_PASS : flag, phases = 0, no_roots = 0;
     if (a.pre && initial > 0) {
         phases = 1;
         if (leader) {
@@ -603,7 +605,7 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         n_free -= eps;
     }
     // ---- results: every block its own words
-    if (status >= 0) {
+    if (status >= 0 && status != SOLO_PASS) {
         for (int w = rank + C * warp; w < (nr + 31) >> 5; w += C * (T / 32)) {
             const int r = w * 32 + lane;
             if (r < nr) {
@@ -668,7 +670,7 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
 // more than GREEDY_LIGHT rows a warp each from the block's list.  Adds to the
 // installed matching; |M| goes to the control block and the host's copy.
 template <int C, int T>
-__global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* __restrict__ rdeg, Ctl* h_ctl) {
+__global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* __restrict__ rdeg, Ctl* h_ctl, int check_err) {
     using namespace bmd;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ int s_card, s_long;
@@ -678,6 +680,9 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     const unsigned s_state = saddr(state);
     const int own_tiles = (((nc + 31) >> 5) + C - 1) / C;
     int32_t* const longs = (int32_t*)p.queue + rank * own_tiles * 32;  // (the queue holds 2 nc words)
+    // an invalid CSR is not read (the same in every block: only the last statement writes the word)
+    const int err = check_err ? ld_volatile(&p.ctl->err) : 0;
+    if (err != 0) return;
     if (t == 0) s_card = s_long = 0;
     __syncthreads();
     int n = 0;

@@ -906,19 +906,43 @@ int grid_for(bm_ctx* ctx, int n) {  // plain launches: enough blocks to fill the
 // 127; 10,000 rows (45 k) 374 / - / 215; 20,000 rows 344 / - / 205; 60,000 rows 463 / - / 391, but 551 / - /
 // 662 for its search from the empty matching, whose levels are wide.
 constexpr int kSoloBlocks = 16;
-constexpr int64_t kSoloOneBlock = 8192;    // entries up to which one block is faster than 16
-constexpr int32_t kSoloMaxSide = 32768;    // rows and columns up to which 16 blocks are faster than the grid
-constexpr int64_t kSoloMaxEdges = 393216;  // ... and entries (8 MB of L2-resident rows is the grid's)
+// One block up to so many entries and columns (5,000 columns of a row each, search from nothing: one block
+// 57 us, grid 42 us), and for fewer columns than 16 blocks own (32 each) up to more entries: 500 columns of
+// 200 rows, 100 k entries, search from nothing 145 us on one block, 106 us on the grid, 50 k entries 113 / 80 us,
+// 32 k entries 75 / 105 us.
+constexpr int64_t kSoloOneBlock = 8192;
+constexpr int32_t kSoloOneBlockCols = 4096;
+constexpr int64_t kSoloOneBlockDense = 32768;
+// 16 blocks for the search up to so many rows, columns and entries (390 k entries of 19,500 columns 106 us, grid
+// 139 us), but of more columns than rows, most of whose trees are searched in vain, not many columns with many
+// entries: 24,000 columns of 19,200 rows 79 / 71 us at 200 k entries, 19,500 of 15,600 87 / 59 us at 390 k.
+constexpr int32_t kSoloMaxSide = 32768;
+constexpr int64_t kSoloMaxEdges = 393216;
+constexpr int64_t kSoloWideEdges = 196608;
+constexpr int32_t kSoloWideCols = 12288;
+// The cheap matching up to so many entries: 50 us on both at 100 k, 59 / 51 us at 150 k, 117 / 78 us at 390 k.
+constexpr int64_t kSoloMaxGreedy = 98304;
+// A path's end and every step back from it write to all 16 blocks, so from more unmatched columns than this the
+// search is left to the grid: the 30,000 x 30,000 identity from a given empty matching 150 us there, now 74 us
+// (a launch that finds out included), 13,000 columns of 20 of 16,250 rows 160 / 111 us, but 10,700 of 3 175 / 255 us.
+constexpr int32_t kSoloMaxRoots = 12288;
+static_assert(kSoloMaxSide <= bms1::SOLO_MAX, "16-bit ids");
 
 int solo_cluster(const bm_ctx* ctx) {
     if (ctx->nr > kSoloMaxSide || ctx->nc > kSoloMaxSide || ctx->nnz > kSoloMaxEdges || ctx->opt.block_size != 0 ||
         ctx->opt.blocks_per_sm != 0 || ctx->opt.deterministic)
         return 0;
-    const int C = ctx->nnz > kSoloOneBlock && ctx->nc >= 32 * kSoloBlocks ? kSoloBlocks : 1;
+    if (ctx->nc > ctx->nr && ctx->nnz > kSoloWideEdges && ctx->nc > kSoloWideCols) return 0;
+    const bool narrow = ctx->nc < 32 * kSoloBlocks;
+    if (narrow && ctx->nnz > kSoloOneBlockDense) return 0;
+    const int C = narrow || (ctx->nnz <= kSoloOneBlock && ctx->nc <= kSoloOneBlockCols) ? 1 : kSoloBlocks;
     if (C > 1 && !ctx->solo_clusters) return 0;
     if (bms1::Layout(ctx->nr, ctx->nc, ctx->nnz, C).bytes > (unsigned)bms1::SOLO_SMEM) return 0;
     return C;
 }
+
+// The cheap matching runs there too.
+bool solo_greedy(const bm_ctx* ctx) { return ctx->nnz <= kSoloMaxGreedy && solo_cluster(ctx) > 0; }
 
 void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* at, int C, size_t smem, cudaStream_t st) {
     cfg.gridDim = dim3((unsigned)C);
@@ -1190,18 +1214,25 @@ int32_t ensure_det_arena(bm_ctx* ctx) {
     return BM_OK;
 }
 
+// The cheap matching on the grid (launch_greedy) of the context's graph and matching.
+int32_t run_greedy(bm_ctx* ctx, bool clear) {
+    const int32_t rc = ensure_rdeg(ctx);
+    if (rc) return rc;
+    launch_greedy(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, clear, ctx->classes,
+                  ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, ctx->stream);
+    BM_CUDA(ctx, cudaGetLastError());
+    return BM_OK;
+}
+
 // Runs the method (or one BFS) on the installed matching.  The control block
 // is cleared by the caller beforehand so that input checks queued before can
 // report through it.
 int32_t run(bm_ctx* ctx, bool bfs_only) {
     Params p = make_params(ctx, bfs_only);
     if (!bfs_only && starts_cheap(ctx)) {
-        const int32_t rc = ensure_rdeg(ctx);
+        const int32_t rc = run_greedy(ctx, false);
         if (rc) return rc;
-        // (its list counters are two of the queue counters, which the matching kernel needs at zero)
-        launch_greedy(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, false,
-                      ctx->classes, ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, ctx->stream);
-        BM_CUDA(ctx, cudaGetLastError());
+        // its list counters are two of the queue counters, which the matching kernel needs at zero
         BM_CUDA(ctx, cudaMemsetAsync(&ctx->ctl->qcnt[0], 0, 2 * sizeof(int32_t), ctx->stream));
         p.pre = 1;
     }
@@ -1288,26 +1319,28 @@ bool solo_match(const bm_ctx* ctx) {
 }
 
 // The cheap matching on one block or cluster; |M| is in ctx->h_ctl when the stream has been waited for.
-int32_t run_solo_greedy(bm_ctx* ctx) {
+// check_err: after input checks that report through the control block.
+int32_t run_solo_greedy(bm_ctx* ctx, bool check_err) {
     const int32_t rc = ensure_rdeg(ctx);
     if (rc) return rc;
     const int C = solo_cluster(ctx);
     const size_t smem = 128 * ((((size_t)ctx->nr + 31) / 32 + C - 1) / C);
     BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo_greedy<1, bms1::SOLO_T1> : bms1::k_solo_greedy<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream,
-                          make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl));
+                          make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl, check_err ? 1 : 0));
     return BM_OK;
 }
 
 // The whole search on one block from (rm_src, cm_src); the outcome is in
 // ctx->h_ctl when the stream has been waited for.
 int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool check_src, bool check_err,
-                 int32_t* rm_out, int32_t* cm_out, int32_t* card_out, bm_stats* stats) {
+                 int32_t* rm_out, int32_t* cm_out, int32_t* card_out, bm_stats* stats, bool* pass) {
+    *pass = false;
     const Params p = make_params(ctx, false);
-    // (the cheap matching's kernel clears the control block, so not after input checks that report through it)
-    const bool pre = !check_src && !check_err && starts_cheap(ctx);
-    const bms1::SoloArgs a{rm_src, cm_src, rm_out, cm_out, ctx->h_ctl, check_src ? 1 : 0, check_err ? 1 : 0, pre ? 1 : 0};
+    const bool pre = !check_src && starts_cheap(ctx);
+    const bms1::SoloArgs a{rm_src, cm_src, rm_out, cm_out, ctx->h_ctl, check_src ? 1 : 0, check_err ? 1 : 0, pre ? 1 : 0,
+                            pre ? 0x7fffffff : kSoloMaxRoots};
     if (pre) {
-        const int32_t rc = run_solo_greedy(ctx);
+        const int32_t rc = solo_greedy(ctx) ? run_solo_greedy(ctx, check_err) : run_greedy(ctx, !check_err);
         if (rc) return rc;
     }
     ctx->empty = false;
@@ -1316,6 +1349,11 @@ int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool
     BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo<1, bms1::SOLO_T1> : bms1::k_solo<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream, p, a,
                                 (long long)ctx->nnz));
     BM_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    if (ctx->h_ctl->status == bms1::SOLO_PASS) {
+        BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), ctx->stream));
+        *pass = true;
+        return BM_OK;
+    }
     return report(ctx, true, card_out, stats);
 }
 
@@ -1510,8 +1548,8 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
     if (ctx->sticky || !ctx->csr_ready) return BM_ERR_STATE;
     cudaStream_t st = ctx->stream;
     ctx->empty = false;
-    if (solo_cluster(ctx) > 0) {
-        const int32_t rc = run_solo_greedy(ctx);
+    if (solo_greedy(ctx)) {
+        const int32_t rc = run_solo_greedy(ctx, false);
         if (rc) return rc;
         BM_CUDA(ctx, cudaStreamSynchronize(st));
         if (card_out) *card_out = ctx->h_ctl->card;
@@ -1530,11 +1568,8 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         k_count_matched<<<grid_for(ctx, ctx->nc), ctx->block, 0, st>>>(ctx->nc, ctx->cmatch, ctx->ctl);
         BM_CUDA(ctx, cudaGetLastError());
     } else if (ctx->nc) {
-        const int32_t rc = ensure_rdeg(ctx);
+        const int32_t rc = run_greedy(ctx, true);
         if (rc) return rc;
-        launch_greedy(ctx->nr, ctx->nc, ctx->nnz, ctx->col_ptr, ctx->row_idx, ctx->rmatch, ctx->cmatch, ctx->ctl, true, ctx->classes,
-                      ctx->rdeg, ctx->endpoints, (int32_t*)ctx->queue, grid_cap(ctx), ctx->block, st);
-        BM_CUDA(ctx, cudaGetLastError());
     }
     int32_t rc = sync_ctl(ctx);
     if (rc) return rc;
@@ -1584,8 +1619,11 @@ int32_t bm_match(bm_ctx* ctx, int32_t* rmatch_out, int32_t* cmatch_out, int32_t*
     bmi::NvtxRange nvtx_range("bm_match");
     if (!ctx) return BM_ERR_INVALID_ARG;
     if (ctx->sticky || !ctx->csr_ready) return BM_ERR_STATE;
-    if (solo_match(ctx))
-        return run_solo(ctx, ctx->rmatch, ctx->cmatch, false, false, rmatch_out, cmatch_out, card_out, stats);
+    if (solo_match(ctx)) {
+        bool pass;
+        const int32_t rc1 = run_solo(ctx, ctx->rmatch, ctx->cmatch, false, false, rmatch_out, cmatch_out, card_out, stats, &pass);
+        if (!pass) return rc1;
+    }
     cudaStream_t st = ctx->stream;
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     int32_t rc = run(ctx, false);
@@ -1602,13 +1640,16 @@ int32_t bm_match_from(bm_ctx* ctx, const int32_t* rmatch0, const int32_t* cmatch
     if (ctx->sticky || !ctx->csr_ready) return BM_ERR_STATE;
     ctx->empty = false;
     if (solo_match(ctx)) {
-        const int32_t rc1 = run_solo(ctx, rmatch0, cmatch0, true, false, rmatch_out, cmatch_out, card_out, stats);
-        if (rc1 != BM_ERR_INVALID_MATCHING) return rc1;
-        ctx->sticky = 0;  // bad input is not a broken context: leave the empty matching installed
-        const int32_t rc2 = clear_matching(ctx);
-        if (rc2) return rc2;
-        cudaStreamSynchronize(ctx->stream);
-        return rc1;
+        bool pass;
+        const int32_t rc1 = run_solo(ctx, rmatch0, cmatch0, true, false, rmatch_out, cmatch_out, card_out, stats, &pass);
+        if (!pass) {
+            if (rc1 != BM_ERR_INVALID_MATCHING) return rc1;
+            ctx->sticky = 0;  // bad input is not a broken context: leave the empty matching installed
+            const int32_t rc2 = clear_matching(ctx);
+            if (rc2) return rc2;
+            cudaStreamSynchronize(ctx->stream);
+            return rc1;
+        }
     }
     cudaStream_t st = ctx->stream;
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
@@ -1638,11 +1679,14 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
         return BM_ERR_INVALID_ARG;
     if (ctx->sticky || !ctx->owns_csr) return BM_ERR_STATE;
     cudaStream_t st = ctx->stream;
+    bool solo = solo_match(ctx);
     BM_CUDA(ctx, cudaMemsetAsync(ctx->ctl, 0, sizeof(Ctl), st));
     BM_CUDA(ctx, cudaMemcpyAsync((void*)ctx->col_ptr, h_col_ptr, 4 * ((size_t)ctx->nc + 1), cudaMemcpyHostToDevice, st));
     if (ctx->nnz)
         BM_CUDA(ctx, cudaMemcpyAsync((void*)ctx->row_idx, h_row_idx, 4 * (size_t)ctx->nnz, cudaMemcpyHostToDevice, st));
-    ctx->empty = h_rmatch == nullptr;
+    // (a small graph's given arrays are looked through: most often they are there to take the result.  An entry in
+    // h_cmatch alone is found by the check below, which stops the launches.)
+    ctx->empty = h_rmatch == nullptr || (solo && std::all_of(h_rmatch, h_rmatch + ctx->nr, [](int32_t c) { return c == -1; }));
     if (h_rmatch) {
         if (ctx->nr) BM_CUDA(ctx, cudaMemcpyAsync(ctx->rmatch, h_rmatch, 4 * (size_t)ctx->nr, cudaMemcpyHostToDevice, st));
         if (ctx->nc) BM_CUDA(ctx, cudaMemcpyAsync(ctx->cmatch, h_cmatch, 4 * (size_t)ctx->nc, cudaMemcpyHostToDevice, st));
@@ -1652,8 +1696,7 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
     }
     // input checks report through the control block; the match launch then
     // returns at once if one failed
-    const bool solo = solo_match(ctx);
-    int32_t rc = validate_csr_async(ctx, !solo && starts_cheap(ctx));
+    int32_t rc = validate_csr_async(ctx, starts_cheap(ctx));
     if (rc) return rc;
     k_check_matching<<<grid_for(ctx, ctx->nr > ctx->nc ? ctx->nr : ctx->nc), ctx->block, 0, st>>>(ctx->nr, ctx->nc, ctx->rmatch, ctx->cmatch, ctx->ctl);
     BM_CUDA(ctx, cudaGetLastError());
@@ -1665,9 +1708,12 @@ int32_t bm_match_host(bm_ctx* ctx, const int32_t* h_col_ptr, const int32_t* h_ro
         if (ctx->h_ctl->err) { ctx->csr_ready = false; return ctx->h_ctl->err; }
     }
     if (solo) {
-        rc = run_solo(ctx, ctx->rmatch, ctx->cmatch, false, true, nullptr, nullptr, card_out, stats);
+        bool pass;
+        rc = run_solo(ctx, ctx->rmatch, ctx->cmatch, false, true, nullptr, nullptr, card_out, stats, &pass);
+        solo = !pass;
         if (rc < 0 && rc != BM_ERR_INVALID_CSR && rc != BM_ERR_INVALID_MATCHING) return rc;
-    } else {
+    }
+    if (!solo) {
         rc = run(ctx, false);
         if (rc < 0) return rc;
     }

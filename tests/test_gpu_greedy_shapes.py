@@ -1,13 +1,14 @@
 """The cheap matching on graphs of extreme shapes: few columns of many rows and
 the reverse, single degree classes, rows that all columns list, rows whose
-entry counts share a slot, diagonals, hubs."""
+entry counts share a slot, diagonals, hubs, and both sides of the limits that
+send a graph to one block, a cluster of blocks or the grid."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_1303_1379_gb300 import bmatch, synth
 
-from helpers import oracle_max, to_dev
+from helpers import assert_maximum, oracle_max, to_dev
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -169,3 +170,84 @@ def test_first_phase_from_nothing(shape):
     want = oracle_max(g)
     assert res.card == want == ends.sum() == res.stats["endpoints"] and res.stats["initial_card"] == 0
     assert ends[0] > 0.5 * want and levels.sum() == res.stats["levels"]
+
+
+ROUTES = {  # rows, columns, entries a column -> blocks of the search (0: the grid)
+    (64, 64, 10): 1, (1024, 1024, 8): 1, (1100, 1025, 8): 16, (20000, 4096, 2): 1, (20000, 4097, 1): 16,
+    (3000, 511, 64): 1, (3000, 511, 65): 0, (3000, 512, 65): 16,
+    (32768, 32768, 6): 16, (32768, 32768, 12): 16, (32768, 32768, 13): 0, (32769, 100, 3): 0, (100, 32769, 3): 0,
+    (12000, 12288, 17): 16, (12000, 12289, 17): 0, (12000, 12288, 16): 16, (16000, 16384, 12): 16,
+}
+
+
+@pytest.mark.parametrize("shape", list(ROUTES), ids=str)
+def test_routes_of_small_graphs(shape):
+    """Every call on both sides of the limits, the result checked and the route read from the statistics."""
+    nr, nc, k = shape
+    rng = np.random.default_rng(k)
+    base = rng.permutation(nr)
+    lists = [base[(c * 37 + np.arange(k) * (1 + c % 5)) % nr] for c in range(nc)]
+    g = from_lists(nr, lists)
+    want = oracle_max(g)
+    cp, ri = to_dev(g)
+    r0, c0, _ = oracle.greedy(nr, nc, g.col_ptr, g.row_idx)
+    rm = torch.empty(nr, dtype=torch.int32, device="cuda")
+    cm = torch.empty(nc, dtype=torch.int32, device="cuda")
+
+    def check(res, a, b):
+        assert_maximum(g, a.cpu().numpy() if torch.is_tensor(a) else a, b.cpu().numpy() if torch.is_tensor(b) else b, res.card, want)
+        assert res.stats["grid"] == ROUTES[shape] or (not ROUTES[shape] and res.stats["grid"] > 16)
+        assert res.stats["endpoints"] == want - res.stats["initial_card"]
+
+    with bmatch.Matcher(nr, nc, g.nnz, cp, ri) as m:
+        check(m.match(rm, cm), rm, cm)  # from nothing
+        m.set_matching()
+        m.greedy()
+        check(m.match(rm, cm), rm, cm)
+        check(m.match_from(torch.from_numpy(r0).cuda(), torch.from_numpy(c0).cuda(), rm, cm), rm, cm)
+    with bmatch.Matcher(nr, nc, g.nnz) as m:
+        h_r, h_c = np.full(nr, -1, np.int32), np.full(nc, -1, np.int32)
+        check(m.match_host(g.col_ptr, g.row_idx, h_r, h_c), h_r, h_c)  # given, but empty
+        assert m.match_host(g.col_ptr, g.row_idx).card == want
+        h_r, h_c = r0.copy(), c0.copy()
+        check(m.match_host(g.col_ptr, g.row_idx, h_r, h_c), h_r, h_c)
+        # an entry of the columns' array alone is not an empty start, and a bad row is not read
+        h_r, h_c = np.full(nr, -1, np.int32), np.full(nc, -1, np.int32)
+        h_c[nc // 2] = 0
+        with pytest.raises(bmatch.BMError) as e:
+            m.match_host(g.col_ptr, g.row_idx, h_r, h_c)
+        assert e.value.status == bmatch.BM_ERR_INVALID_MATCHING
+        bad = g.row_idx.copy()
+        bad[g.nnz // 2] = nr
+        for given in ((), (np.full(nr, -1, np.int32), np.full(nc, -1, np.int32))):
+            with pytest.raises(bmatch.BMError) as e:
+                m.match_host(g.col_ptr, bad, *given)
+            assert e.value.status == bmatch.BM_ERR_INVALID_CSR
+        assert m.match_host(g.col_ptr, g.row_idx).card == want
+
+
+@pytest.mark.parametrize("n", [12288, 12289])
+@pytest.mark.parametrize("call", ["from", "host", "installed"])
+def test_many_unmatched_columns_go_to_the_grid(n, call):
+    """A given start that leaves more columns unmatched than the cluster searches from; one more pair is matched."""
+    nr = n + 1
+    g = from_lists(nr, [[c, (c + 1) % nr] for c in range(n + 1)])
+    rm, cm = np.full(nr, -1, np.int32), np.full(n + 1, -1, np.int32)
+    rm[0], cm[n] = n, 0
+    cp, ri = to_dev(g)
+    d_rm, d_cm = torch.from_numpy(rm).cuda(), torch.from_numpy(cm).cuda()
+    with bmatch.Matcher(nr, n + 1, g.nnz) as m:
+        if call == "host":
+            res = m.match_host(g.col_ptr, g.row_idx, rm, cm)
+        else:
+            m.upload_csr(g.col_ptr, g.row_idx)
+            if call == "installed":
+                m.set_matching(d_rm, d_cm)
+                res = m.match(d_rm, d_cm)
+            else:
+                res = m.match_from(d_rm, d_cm, d_rm, d_cm)  # in place
+            rm, cm = d_rm.cpu().numpy(), d_cm.cpu().numpy()
+        assert_maximum(g, rm, cm, res.card, n + 1)
+        assert res.stats["initial_card"] == 1 and (res.stats["grid"] == 16) == (n <= 12288)
+        again = m.match()
+        assert again.card == n + 1 and again.stats["initial_card"] == n + 1
