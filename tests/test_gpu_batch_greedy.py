@@ -67,3 +67,25 @@ def test_batch_default_geometry(n, block):
     for k in (0, n - 1):
         g = graphs[k]
         assert int(card[k]) == oracle.hopcroft_karp(g.n_rows, g.n_cols, g.col_ptr, g.row_idx)[2]
+
+
+@pytest.mark.parametrize("first", [{"deterministic": 1}, {"bfs": 0}, {"wr_one_endpoint": 0}], ids=str)
+def test_batch_counts_rows_when_an_option_comes_to_read_them(first):
+    """Created with options that do not read the rows' entry counts, matched with ones that do: a column lists a row
+    of everyone's, one shared with few and one of its own, which the cheap matching must give it."""
+    n = 3000  # (no row has its column's number)
+    lists = [np.roll([n, n + 1 + c % 100, n + 101 + c], c % 3) for c in range(n)]
+    one = synth.Graph(2 * n + 101, n, (3 * np.arange(n + 1)).astype(np.int32), np.concatenate(lists).astype(np.int32), "own rows")
+    b = to_batch([one, synth.uniform_graph(70000, 300, 4, seed=1), one])
+    with bmatch.Batch.from_synth(b, **first) as bb:
+        rm = torch.full((int(b.row_off[-1]),), -1, dtype=torch.int32, device="cuda")
+        cm = torch.full((int(b.col_off[-1]),), -1, dtype=torch.int32, device="cuda")
+        bb.match(rm, cm)
+        assert int((cm >= 0).sum()) == 2 * n + 300
+        bb.set_options(deterministic=0, bfs=1, wr_one_endpoint=1)
+        rm.fill_(-1)
+        cm.fill_(-1)
+        bb.match(rm, cm)
+    for k in (0, 2):
+        assert np.array_equal(cm[b.col_off[k]:b.col_off[k + 1]].cpu().numpy(), n + 101 + np.arange(n))
+    assert int((cm >= 0).sum()) == 2 * n + 300
