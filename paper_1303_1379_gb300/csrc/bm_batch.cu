@@ -13,8 +13,10 @@
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <numeric>
+#include <queue>
 #include <vector>
 
 #include "bm_device.cuh"
@@ -197,7 +199,9 @@ __global__ void k_batch_rdeg8(long long n, const int32_t* rdeg, uint8_t* rdeg8) 
 struct bm_batch {
     bm_batch_desc d{};
     bool rdeg_ready = false;  // rdeg8 holds the rows' entry counts
-    int64_t total_rows = 0, total_cols = 0, total_edges = 0, max_edges = 0;
+    int64_t total_rows = 0, total_cols = 0, total_edges = 0;
+    std::vector<int64_t> edges;  // the graphs' entries, most first
+    int l2_bytes = 0;
     cudaStream_t stream = nullptr;
     bm_options opt{};
     int block = 512, grid = 0, num_sms = 0;
@@ -268,6 +272,48 @@ BatchParams batch_params(bm_batch* b, int32_t* rmatch, int32_t* cmatch, int gree
     return bp;
 }
 
+// How long `slots` blocks take that draw graphs largest first: edges, sorted so, a graph costing fixed + slope
+// times its entries.
+double launch_estimate(const std::vector<int64_t>& edges, int slots, double slope) {
+    constexpr double fixed = 16000;
+    double sum = 0;
+    for (int64_t e : edges) sum += fixed + slope * (double)e;
+    if ((int64_t)edges.size() > 4 * (int64_t)slots)  // the sum is what counts
+        return std::max(sum / slots, fixed + slope * (double)edges[0]);
+    std::priority_queue<double, std::vector<double>, std::greater<double>> free_at;
+    double end = 0;
+    for (int64_t e : edges) {
+        double t = fixed + slope * (double)e;
+        if ((int)free_at.size() == slots) {
+            t += free_at.top();
+            free_at.pop();
+        }
+        free_at.push(t);
+        end = std::max(end, t);
+    }
+    return end;
+}
+
+// Whether a batch whose caller leaves the launch to the library gets one block of 1,024 threads an SM (else two of
+// 512).  The wider block is the faster one for a graph by itself, by the more the larger the graph, and for the
+// smallest no faster; but there are half as many.  So both launches are estimated from the graphs' entries: a graph
+// takes about as long as 16,000 entries more than it has (a few dozen barriers), and 1.8 times as long per entry on
+// the narrower of two blocks an SM (2.3 times with the deterministic option and more data than L2 holds, about 28
+// bytes a row and a column and 4 an entry).  One GB300, ms at 512 / 1,024 threads, default and deterministic:
+// graphs of 100 to 50,000 rows, 48 of them 1.31 / 0.97, 3.97 / 2.38; 512 2.17 / 1.40, 6.7 / 4.8; 2,048 3.0 / 2.7,
+// 15.2 / 11.7; 4,096 4.86 / 5.00; equal graphs of 1,000 rows, 152 of them 0.168 / 0.167, 0.48 / 0.42; 200 0.169 /
+// 0.236, 0.46 / 0.62; 400 0.23 / 0.32, 0.72 / 0.91; of 20,000 rows, 100 0.92 / 0.55, 3.1 / 2.1; 200 1.08 / 1.03, 5.0
+// / 4.5; 400 1.9 / 1.55, 10.4 / 7.6; one of 50,000 rows and 1,000 of 200 2.0 / 1.4, 4.9 / 3.5, and 8,000 of 200 2.1 /
+// 2.6, 6.0 / 7.0; 300 meshes of 60 x 60 0.72 / 0.88, 3.5 / 5.7.
+bool wide_blocks(const bm_batch* b) {
+    const int64_t n = (int64_t)b->edges.size();
+    if (n <= b->num_sms) return n > 0;
+    const double at_once = std::min(1.0, 2.0 * b->num_sms / (double)n);  // part of the batch on the chip
+    const bool spills = at_once * (28.0 * (double)(b->total_rows + b->total_cols) + 4.0 * (double)b->total_edges) > b->l2_bytes;
+    return launch_estimate(b->edges, b->num_sms, 1.0) <=
+           launch_estimate(b->edges, 2 * b->num_sms, b->opt.deterministic && spills ? 2.3 : 1.8);
+}
+
 // The entry counts are read by the cheap matching of the default routine (block_greedy_sb).
 bool reads_counts(const bm_options& o) { return !o.deterministic && o.bfs == BM_GPUBFS_WR && o.wr_one_endpoint == 1; }
 
@@ -287,13 +333,7 @@ void check_batch(bm_batch* b, bool count) {
 }
 
 int32_t configure_batch(bm_batch* b) {
-    // Without a size from the caller: two blocks of 512 threads an SM while the whole batch is what takes
-    // the time, one of 1,024 when the largest graphs are (they run first, on a block each, and the launch
-    // lasts as long as they do): one GB300, graphs of 100 to 50,000 rows, ms at 512 / 1,024 threads: 512
-    // graphs 2.46 / 1.59, 1,024 2.9 / 2.2, 2,048 3.5 / 3.1, 4,096 4.86 / 5.00; 48 from the empty matching
-    // 2.35 / 1.41.  4,096 such graphs hold 2.3 times num_sms x the largest one's entries, 2,048 half that.
-    const bool few = b->total_edges < 2 * (int64_t)b->num_sms * b->max_edges;
-    b->block = b->opt.block_size ? b->opt.block_size : few && b->opt.blocks_per_sm == 0 ? 1024 : 512;
+    b->block = b->opt.block_size ? b->opt.block_size : b->opt.blocks_per_sm == 0 && wide_blocks(b) ? 1024 : 512;
     int per_sm = 0;
     cudaError_t e = b->opt.deterministic
                         ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch<true, true>, b->block, 0)
@@ -385,12 +425,14 @@ int32_t bm_batch_create(const bm_batch_desc* desc, void* stream, const bm_option
     b->total_rows = ro[G];
     b->total_cols = co[G];
     b->total_edges = eo[G];
-    for (int g = 0; g < G; ++g) b->max_edges = std::max(b->max_edges, eo[g + 1] - eo[g]);
     std::vector<int32_t> order(G);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
         return eo[x + 1] - eo[x] > eo[y + 1] - eo[y];  // most edges first
     });
+    b->edges.resize(G);
+    for (int g = 0; g < G; ++g) b->edges[g] = eo[order[g] + 1] - eo[order[g]];
+    if (cudaDeviceGetAttribute(&b->l2_bytes, cudaDevAttrL2CacheSize, dev) != cudaSuccess) (void)cudaGetLastError();
     auto al = [](size_t v) { return (v + 255) & ~size_t(255); };
     const size_t R = (size_t)(b->total_rows ? b->total_rows : 1), C = (size_t)(b->total_cols ? b->total_cols : 1);
     const size_t G1 = (size_t)(G ? G : 1);

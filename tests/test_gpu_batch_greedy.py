@@ -89,3 +89,28 @@ def test_batch_counts_rows_when_an_option_comes_to_read_them(first):
     for k in (0, 2):
         assert np.array_equal(cm[b.col_off[k]:b.col_off[k + 1]].cpu().numpy(), n + 101 + np.arange(n))
     assert int((cm >= 0).sum()) == 2 * n + 300
+
+
+@pytest.mark.parametrize("sizes,det,block", [
+    # rows x graphs; one block of 1,024 threads an SM holds 152 graphs at once, two of 512 hold 304
+    ([(200, 152)], 0, 1024), ([(200, 153)], 0, 512), ([(200, 303)], 1, 512), ([(1000, 200)], 0, 512),
+    ([(1000, 200)], 1, 512), ([(10000, 1), (200, 600)], 0, 1024), ([(40000, 1), (200, 300)], 0, 1024),
+    ([(40000, 8), (200, 300)], 1, 1024), ([(3000, 20), (100, 280)], 0, 512), ([(20000, 310)], 1, 1024), ([(20000, 310)], 0, 1024),
+], ids=str)
+def test_batch_default_geometry_by_the_longest_wait(sizes, det, block):
+    pool = {nr: synth.uniform_graph(nr, nr + nr // 20, 7, seed=nr) for nr, _ in sizes}
+    graphs = [pool[nr] for nr, n in sizes for _ in range(n)]
+    b = to_batch(graphs)
+    with bmatch.Batch.from_synth(b, deterministic=det) as bb:
+        rm = torch.full((int(b.row_off[-1]),), -1, dtype=torch.int32, device="cuda")
+        cm = torch.full((int(b.col_off[-1]),), -1, dtype=torch.int32, device="cuda")
+        card = torch.empty(len(graphs), dtype=torch.int32, device="cuda")
+        _, st = bb.match(rm, cm, card_out=card)
+        want = {nr: oracle.hopcroft_karp(g.n_rows, g.n_cols, g.col_ptr, g.row_idx)[2] for nr, g in pool.items()}
+        assert card.cpu().tolist() == [want[nr] for nr, n in sizes for _ in range(n)]
+        assert st["block"] == block and st["grid"] == (152 if block == 1024 else 304)
+        # a size from the caller counts as before
+        bb.set_options(blocks_per_sm=1)
+        assert bb.match(rm, cm)[1]["block"] == 512
+        bb.set_options(blocks_per_sm=0, block_size=256)
+        assert bb.match(rm, cm)[1]["block"] == 256
