@@ -33,7 +33,7 @@ namespace {
 constexpr int kVersion = 1 * 10000 + 0 * 100 + 0;
 constexpr int kDefaultBlock = 512;
 constexpr int kProfileCap = 4096;
-constexpr int64_t kDetOneBlockEdges = 4 << 20;  // see configure
+constexpr int64_t kDetOneBlockEdges = 1200 << 10;  // see configure
 
 // ------------------------------------------------------------------ kernels
 
@@ -1003,9 +1003,12 @@ int32_t configure(bm_ctx* ctx) {
         if (per_sm < 1 || per_sm * ctx->num_sms > 2047) return BM_ERR_UNSUPPORTED;
         ctx->coop_grid[wr] = per_sm * ctx->num_sms;
     }
-    // The deterministic search of a graph of up to 4 M entries: one block an SM.  Its levels wait on the grid
-    // barrier and on chains of loads, not for throughput (ms at two / one: permuted 500 x 500 mesh 4.29 / 4.13,
-    // 500 x 500 mesh 79.3 / 74.8, 300 k uniform graph 1.32 / 1.30, but R-MAT 1 M, 13 M entries, 1.19 / 1.32).
+    // The deterministic search of a graph of up to 1.2 M entries: one block an SM.  Its levels wait on the grid
+    // barrier and on chains of loads, not for throughput; with more entries the wide levels of all graphs but meshes
+    // want the threads (time at one block an SM / at two, from the cheap matching: 300 k entries of 100 k columns 0.95,
+    // 400 k 0.92, 600 k 0.96 to 0.98, permuted meshes of 0.1 / 0.4 / 1.2 M entries 0.92 / 0.96 / 0.94, R-MAT of 0.9 M
+    // 0.95; 1.2 M entries of 100 k / 200 k / 400 k columns 1.02 / 1.07 / 1.05; 2.4 M 1.16 to 1.18, 3 M 1.10 to 1.12,
+    // 4 M 1.26, R-MAT of 3.9 M 1.04, permuted mesh of 3.8 M 0.97).
     if (ctx->opt.block_size == 0 && ctx->opt.blocks_per_sm == 0 && ctx->nnz <= kDetOneBlockEdges &&
         ctx->coop_grid[2] > ctx->num_sms)
         ctx->coop_grid[2] = ctx->num_sms;

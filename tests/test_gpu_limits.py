@@ -80,3 +80,22 @@ def test_limited_phases_from_the_empty_matching(block, phases):
     rm, cm = rm.cpu().numpy(), cm.cpu().numpy()
     assert np.all(rm[g.row_idx[np.repeat(cm < 0, np.diff(g.col_ptr))]] >= 0)
     assert res.status == bmatch.BM_INCOMPLETE
+
+
+@pytest.mark.parametrize("nnz,per_sm", [(1200 * 1024, 1), (1200 * 1024 + 1, 2)])
+def test_default_grid_of_the_deterministic_search(nnz, per_sm):
+    """One block an SM up to 1,228,800 entries, two beyond; the matching is the same for every grid."""
+    rng = np.random.default_rng(4)
+    nr, nc = 300000, 200000
+    ptr = np.concatenate([[0], np.sort(rng.integers(0, nnz + 1, nc - 1)), [nnz]]).astype(np.int32)
+    cp, ri = torch.from_numpy(ptr).cuda(), torch.from_numpy(rng.integers(0, nr, nnz).astype(np.int32)).cuda()
+    out = []
+    for options in ({}, {"blocks_per_sm": 3 - per_sm}):
+        rm = torch.empty(nr, dtype=torch.int32, device="cuda")
+        with bmatch.Matcher(nr, nc, nnz, cp, ri, deterministic=1, **options) as m:
+            m.greedy()
+            res = m.match(rm)
+        out.append((rm, res.stats["grid"]))
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert [grid for _, grid in out] == [per_sm * sms, (3 - per_sm) * sms]
+    assert torch.equal(out[0][0], out[1][0])
