@@ -108,7 +108,8 @@ struct alignas(128) Ctl {
                                // here (odd ones in ep_phase), so that each phase's counter can be
                                // cleared during the phase before it
     int32_t classes;           // CSR check: the degree classes that some column is of (greedy_class)
-    int32_t pad1[5];
+    int32_t checks;            // range-checked build: times that the whole matching was checked
+    int32_t pad1[4];
     long long levels;
     long long max_levels;
     long long cols_expanded;
@@ -1547,6 +1548,7 @@ __device__ __forceinline__ void step_check_matching(const Params& p) {
         if (m != -1 && (m < 0 || m >= p.nr || __ldcg(&p.rmatch[m]) != c)) bad = true;
     }
     if (bad && p.chk) atomicCAS(p.chk, 0, -11 /*BM_ERR_CHECK*/);
+    if (tid == 0) ++p.ctl->checks;
 }
 
 // Gives back the rows a BFS-only pass claimed (inspection entry point).

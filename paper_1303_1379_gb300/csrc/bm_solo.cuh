@@ -398,7 +398,10 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         unsigned got[SOLO_U];
         bool ask[SOLO_U], any_free = false;
 #pragma unroll
-        for (int u = 0; u < SOLO_U; ++u) m[u] = own[u] >= 0 ? ((volatile u16*)rm)[r[u]] : -1;
+        for (int u = 0; u < SOLO_U; ++u) {
+            m[u] = own[u] >= 0 ? ((volatile u16*)rm)[r[u]] : -1;
+            if (m[u] >= 0 && m[u] != SOLO_FREE && !bmd::idx_ok(p, m[u], nc)) m[u] = -1;  // checked build only
+        }
 #pragma unroll
         for (int u = 0; u < SOLO_U; ++u) {
             const bool matched = m[u] >= 0 && m[u] != SOLO_FREE;
@@ -457,6 +460,27 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         }
     };
 
+#ifdef BM_CHECKED
+    // Between phases, as step_check_matching: this block's copy of the rows' matches against the columns', wherever
+    // they are, and its own columns' against the copy.  The next phase's levels write a served root's match.
+    int checks = 0;
+    auto check_matching = [&]() {
+        bool bad = false;
+        for (int r = t; r < nr; r += T) {
+            const int c = rm[r];
+            if (c != SOLO_FREE && (c >= nc || dld16(at<C>(s_cm + 2u * slot_of<C>(c), owner<C>(c))) != r)) bad = true;
+        }
+        for (int ow = warp; ow < (int)lay.own_cw; ow += T / 32) {
+            const int c = (ow * C + rank) * 32 + lane, r = cm[ow * 32 + lane];
+            if (c < nc && r != SOLO_FREE && (r >= nr || rm[r] != c)) bad = true;
+        }
+        if (bad && p.chk) atomicCAS(p.chk, 0, -11 /*BM_ERR_CHECK*/);
+        ++checks;
+        __syncthreads();
+        cluster_sync<C>();
+    };
+#endif
+
     while (status == 0) {
         if (n_roots == 0) { no_roots = 1; break; }
         if (phases >= p.max_phases) {
@@ -475,11 +499,13 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
                 unsigned e = 0;
                 if (lane < width && g + lane < nl) {
                     const int sl = (int)(list[g + lane] & 0xffffu), off = (int)(list[g + lane] >> 16) * PART;
-                    e = (unsigned)((((sl >> 5) * C + rank) << 5) | (sl & 31)) << 16 | (pr[sl] & 0xffffu);
-                    beg = col_beg[sl] + off;
-                    deg = min(col_deg[sl] - off, PART);
-                    if (bmd::sb_test(srv, (int)(e & 0xffffu))) deg = 0;  // Algorithm 4: root already served
-                    else if (off == 0) ++cols;
+                    if (bmd::idx_ok(p, sl, 32 * lay.own_cw) && bmd::idx_ok(p, pr[sl] & 0xffffu, nc)) {
+                        e = (unsigned)((((sl >> 5) * C + rank) << 5) | (sl & 31)) << 16 | (pr[sl] & 0xffffu);
+                        beg = col_beg[sl] + off;
+                        deg = min(col_deg[sl] - off, PART);
+                        if (bmd::sb_test(srv, (int)(e & 0xffffu))) deg = 0;  // Algorithm 4: root already served
+                        else if (off == 0) ++cols;
+                    }
                 }
                 int incl = deg;
 #pragma unroll
@@ -599,6 +625,9 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         for (int w = t; w < words; w += T) srv[w] = 0u;
         for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += T) rcl[w] = 0u;
         end_step(true);
+#ifdef BM_CHECKED
+        check_matching();
+#endif
         n_front = sum_cnt;
         status = flag;
         n_roots -= eps;
@@ -658,6 +687,9 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
             c.inserted = sm.st.ins;
             c.roots = sm.st.roots;
             c.kernel_ns = (long long)(bmd::globaltimer() - t_start);
+#ifdef BM_CHECKED
+            c.checks = checks;
+#endif
             *p.ctl = c;
             *a.h_ctl = c;
         }
@@ -680,9 +712,10 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     const unsigned s_state = saddr(state);
     const int own_tiles = (((nc + 31) >> 5) + C - 1) / C;
     int32_t* const longs = (int32_t*)p.queue + rank * own_tiles * 32;  // (the queue holds 2 nc words)
-    // an invalid CSR is not read (the same in every block: only the last statement writes the word)
+    // an invalid CSR is not read (the same in every block: nothing writes the word then)
     const int err = check_err ? ld_volatile(&p.ctl->err) : 0;
     if (err != 0) return;
+    if (!check_err && rank == 0 && t == 0) p.ctl->err = 0;
     if (t == 0) s_card = s_long = 0;
     __syncthreads();
     int n = 0;
@@ -697,7 +730,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     // a block's columns: every C-th tile of 32, in a scattered order
     const int bits = own_tiles > 1 ? 32 - __clz(own_tiles - 1) : 0;  // 2^bits >= own_tiles
     auto state_at = [&](int r) { return at<C>(s_state + 4u * slot_of<C>(r), owner<C>(r)); };
-    auto state_of = [&](int r) { return (int)dld32(state_at(r)); };
+    auto state_of = [&](int r) { return idx_ok(p, r, nr) ? (int)dld32(state_at(r)) : GREEDY_TAKEN; };
     auto take = [&](int r, int seen) { return dcas(state_at(r), seen, GREEDY_TAKEN) == seen; };
     const int limit[4] = {0, 2, 8, GREEDY_LIGHT};
     const bool crowded = greedy_crowded(nr, __ldg(&p.col_ptr[nc])), any = crowded && nc > 2LL * nr;
@@ -738,6 +771,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     if (rank == 0 && t == 0) {
         Ctl c{};
         c.card = s_card;
+        c.err = ld_volatile(&p.ctl->err);  // (range-checked build)
         *p.ctl = c;
         *h_ctl = c;
     }

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1276,11 +1277,18 @@ int32_t run(bm_ctx* ctx, bool bfs_only) {
     return BM_OK;
 }
 
+#ifdef BM_CHECKED
+std::atomic<long long> g_checks{0};  // times that a context's launches checked the whole matching between phases
+#endif
+
 // Outcome of the launch whose control block is in ctx->h_ctl; solo: it was k_solo's.
 int32_t report(bm_ctx* ctx, bool solo, int32_t* card_out, bm_stats* stats) {
     const Ctl& h = *ctx->h_ctl;
     const int32_t status = h.status != 0 ? h.status : h.err;
     if (status < 0) ctx->sticky = status;
+#ifdef BM_CHECKED
+    g_checks += h.checks;
+#endif
     if (card_out) *card_out = h.card;
     if (stats) {
         memset(stats, 0, sizeof(*stats));
@@ -1340,7 +1348,7 @@ int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool
     *pass = false;
     const Params p = make_params(ctx, false);
     const bool pre = !check_src && starts_cheap(ctx);
-    const bms1::SoloArgs a{rm_src, cm_src, rm_out, cm_out, ctx->h_ctl, check_src ? 1 : 0, check_err ? 1 : 0, pre ? 1 : 0,
+    const bms1::SoloArgs a{rm_src, cm_src, rm_out, cm_out, ctx->h_ctl, check_src ? 1 : 0, check_err || pre ? 1 : 0, pre ? 1 : 0,
                             pre ? 0x7fffffff : kSoloMaxRoots};
     if (pre) {
         const int32_t rc = solo_greedy(ctx) ? run_solo_greedy(ctx, check_err) : run_greedy(ctx, !check_err);
@@ -1371,6 +1379,11 @@ int32_t clear_matching(bm_ctx* ctx) {
 
 // ------------------------------------------------------------------ C-ABI
 extern "C" {
+
+#ifdef BM_CHECKED
+// Of the range-checked library only (and not in its header): how often the matching was checked so far.
+BM_API int64_t bm_checked_sweeps(void) { return g_checks.load(); }
+#endif
 
 void bm_default_options(bm_options* opt) {
     if (!opt) return;
@@ -1555,6 +1568,7 @@ int32_t bm_greedy(bm_ctx* ctx, int32_t* card_out) {
         const int32_t rc = run_solo_greedy(ctx, false);
         if (rc) return rc;
         BM_CUDA(ctx, cudaStreamSynchronize(st));
+        if (ctx->h_ctl->err) return ctx->sticky = ctx->h_ctl->err;  // range-checked build
         if (card_out) *card_out = ctx->h_ctl->card;
         return BM_OK;
     }
