@@ -211,10 +211,12 @@ BM_API int32_t bm_get_matching(bm_ctx *ctx, int32_t *rmatch_out, int32_t *cmatch
  * maximum matching to rmatch_out (n_rows) / cmatch_out (n_cols) (device,
  * either may be NULL) and |M| to *card_out (host, nullable); *stats (host,
  * nullable) gets counters.  The context keeps the result as its installed
- * matching.  From the empty matching the default mode (APFB, GPUBFS-WR, one
- * endpoint per root) has its first phase end after its first level, in which
- * every path is one edge and which the kernels of bm_greedy run; stats and
- * profile count it as a phase of one level.
+ * matching.  From the empty matching the first phase is one level, in which
+ * every path is one edge.  The default mode (APFB, GPUBFS-WR, one endpoint per
+ * root) lets the kernels of bm_greedy run it, unless there are more than twice
+ * as many columns as rows: phases, levels, endpoints, roots, alternate_steps
+ * and the profile then count it as any phase, columns_expanded, edges_scanned,
+ * edges_to_matched and kernel_ns (and total_timeout_ns) leave it out.
  */
 BM_API int32_t bm_match(bm_ctx *ctx, int32_t *rmatch_out, int32_t *cmatch_out, int32_t *card_out,
                  bm_stats *stats);
@@ -329,7 +331,8 @@ BM_API int32_t bm_batch_set_options(bm_batch *b, const bm_options *opt);
  * (row_off / col_off slices, local ids), the initial matchings on entry (-1
  * for none) and the maximum matchings on return.  greedy != 0 first runs the
  * cheap matching of Section 4 inside the launch (without it, a graph whose
- * initial matching is empty has its first phase cut as in bm_match).  card_out: device
+ * initial matching is empty has it run the first phase, and counted, as in
+ * bm_match).  card_out: device
  * [n_graphs] (nullable) gets each |M|.  Returns the first per-graph error (see
  * bm_batch_graph_status) or BM_OK. */
 BM_API int32_t bm_batch_match(bm_batch *b, int32_t greedy, int32_t *rmatch, int32_t *cmatch,

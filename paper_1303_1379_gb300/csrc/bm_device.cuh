@@ -65,13 +65,13 @@ constexpr int RV_MAX_Q = 32768;  // largest level (columns) that claims through 
 // column has shown the forest closed, as a search from the roots would.  And since a
 // phase that ends early loses nothing, one that has found endpoints ends once its levels
 // are narrow (a few columns a level against the forest: each level is a round trip of the
-// whole grid, and starting the next phase costs about two).
+// whole grid, and ending a phase and starting the next, 13 + 14 us, costs about five).
 // Long augmenting paths do not gain from it: a carried tree's paths are not the shortest.
 // So a search that needs many phases stops cutting them short after CUT_PHASES and starts
 // from its roots again after CARRY_PHASES.  One GB300, search alone, before -> after
-// (phases / levels): 300 k uniform graph 776 -> 465 us (5 / 130 -> 8 / 44); R-MAT 1 M
-// 521 -> 418 us (4 / 44 -> 5 / 22); R-MAT scale 21 786 -> 658 us; 2000 x 2000 mesh 66 -> 57 ms
-// (13 / 11.4 k -> 20 / 9.5 k; 62 ms cut for 6 phases only, 71 ms rebuilt after 10); the mesh
+// (phases / levels): 300 k uniform graph 776 -> 420 us (5 / 130 -> 6 / 55); R-MAT 1 M
+// 521 -> 350 us (4 / 44 -> 4 / 25); R-MAT scale 21 786 -> 605 us; 2000 x 2000 mesh 66 -> 57 ms
+// from a matching without the diagonal's rule (13 / 11.4 k -> 20 / 9.5 k; 62 ms cut for 6 phases only, 71 ms rebuilt after 10); the mesh
 // from the one-sided start of a first-free-row matching 210 -> 201 ms (417 ms if carried to
 // the end).  CUT_MIN 3 to 7 and no ratio are within 5% on the random graphs.
 constexpr int CARRY_PHASES = 20;
@@ -205,7 +205,8 @@ __device__ __forceinline__ unsigned long long globaltimer() {
 }
 
 // A mixing of 32 bits in which every input bit reaches every output bit (two
-// rounds of xor-shift and multiplication by odd constants, a bijection).
+// rounds of xor-shift and multiplication by odd constants, a bijection; the
+// constants here and in scatter_bits are primes that xxHash32 publishes).
 __device__ __forceinline__ unsigned hash32(unsigned x) {
     x ^= x >> 16;
     x *= 0x9e3779b1u;
@@ -237,6 +238,8 @@ __device__ __forceinline__ void set_error(Ctl* ctl, int code) { atomicCAS(&ctl->
 // a queue entry) is checked before it is used; an index out of range records
 // BM_ERR_CHECK (-11) in p.chk and the access is skipped, so a fault in the
 // method's bookkeeping shows as a status instead of a stray memory access.
+// The two searches of the default option (k_match, k_solo) also check between
+// phases that the matching's two arrays are inverse to each other.
 // In the normal build the checks compile to nothing.
 #ifdef BM_CHECKED
 __device__ __forceinline__ bool idx_ok(const Params& p, long long i, long long n) {
@@ -1564,11 +1567,11 @@ __device__ __forceinline__ void step_release_endpoints(const Params& p, int n_ep
 // ------------------------------------------------------------------ one graph, one block
 // The cheap matching of one graph by one block with the rows' marks in shared
 // memory (p.vis: one bit per matched row, at most SB_MAX_COLS rows): the
-// whole-GPU passes' choice (the least-listed free row of a rotated list, columns
-// scattered), but a column looks at GW rows of its list at a time and takes the
-// first window's, and all degrees go in one pass.  A thread takes two columns at
-// a time, their loads in flight together.  (4,096 graphs, ms for the launch: first
-// free row 5.53, this 4.86, shortest lists first in three passes 5.33, four rows a
+// whole-GPU passes' choice (the column's own number, else the least-listed free
+// row of a rotated list, columns scattered), but a column looks at GW rows of its
+// list at a time and takes the first window's, and all degrees go in one pass.  A
+// thread takes two columns at a time, their loads in flight together.  (Without the
+// own number's rule, 4,096 graphs, ms for the launch: first free row 5.53, this 4.86, shortest lists first in three passes 5.33, four rows a
 // window 5.31, columns in order 4.76 -- but 64 meshes of 150 x 150 and more take
 // 16.4 / 3.6 / - / 3.4 / 7.0.)
 template <bool NC>
@@ -1753,7 +1756,8 @@ __device__ int block_match_graph(const Params& p, int greedy, Smem& sm, Counters
     // graphs of 100 to 50,000 rows from the empty matching: 1.43 -> 0.95 ms).
     const bool empty = __syncthreads_or(matched) == 0;
     const bool pre = rows_sb && p.rdeg8 && !greedy && p.mode == 0 && empty;
-    // ---- cheap matching (Section 4): unmatched columns claim their first free row.
+    // ---- cheap matching (Section 4): unmatched columns claim a free row, with the rows' marks and entry
+    // counts by block_greedy_sb's choice, otherwise the first of their list.
     // A thread walks the lists of GU columns together, GW rows of each per step,
     // so that GU x GW row loads (and, without rows_sb, then GU x GW match loads)
     // are in flight at once and a thread takes as long as its longest walk / GW

@@ -1341,8 +1341,8 @@ int32_t run_solo_greedy(bm_ctx* ctx, bool check_err) {
     return BM_OK;
 }
 
-// The whole search on one block from (rm_src, cm_src); the outcome is in
-// ctx->h_ctl when the stream has been waited for.
+// The whole search on one block or cluster from (rm_src, cm_src), with its outcome; *pass: nothing was done, the
+// start leaves more columns unmatched than it searches from (kSoloMaxRoots), and the control block is cleared.
 int32_t run_solo(bm_ctx* ctx, const int32_t* rm_src, const int32_t* cm_src, bool check_src, bool check_err,
                  int32_t* rm_out, int32_t* cm_out, int32_t* card_out, bm_stats* stats, bool* pass) {
     *pass = false;
