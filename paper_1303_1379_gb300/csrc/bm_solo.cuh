@@ -56,6 +56,7 @@ constexpr int SOLO_MAX = 0xfffe;       // rows and columns with a 16-bit id
 constexpr int SOLO_SMEM = 216 * 1024;  // dynamic shared memory of a block
 constexpr int PART = 128;              // a listed column's rows are expanded in parts of this many
 constexpr int SOLO_U = 2;              // edges of a thread in flight
+constexpr int TIMED_OUT = -(1 << 30);  // added to a level's columns: the launch's time is up
 constexpr int SOLO_PASS = 2;           // status: the search is left to the grid
 constexpr int ROW_GLOBAL = 1 << 30;    // marks row positions in the graph's own row_idx
 
@@ -550,10 +551,11 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
             wins = __reduce_add_sync(FULL, wins);
             if (lane == 0 && wins) atomicAdd(&sm.mine.cnt, wins);
             wins = 0;
-            // the launch's limit, at every eighth level: a phase of a long path is thousands of them
-            if (leader && (level & 7) == 0 && bmd::globaltimer() > deadline) sm.mine.flag = -5 /*BM_ERR_TIMEOUT*/;
+            // the launch's limit, after a phase (below) and within it at every 16th level: a long path's are thousands.
+            // It ends the phase in the columns' count, which every block looks at anyway (a flag of its own, read at
+            // each level, cost a search 2%), and the warp that tests it is the last to get columns.
+            if (rank == 0 && t == T - 1 && (level & 15) == 15 && bmd::globaltimer() > deadline) atomicAdd(&sm.mine.cnt, TIMED_OUT);
             end_step(false);
-            if (flag != 0) break;  // the same in every block
             ++level;
             eps += sum_eps;
             if (leader) {
@@ -564,13 +566,13 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
                 }
             }
             tail += sum_cnt;
-            if (sum_cnt == 0) break;  // no vertex inserted
+            if (sum_cnt <= 0) break;  // no vertex inserted, or out of time
             if (carry && eps > 0 && phases <= bmd::CUT_PHASES && level >= bmd::CUT_MIN && level <= bmd::CUT_MAX &&
                 sum_cnt * bmd::CUT_RATIO <= tail)
                 break;
         }
-        if (flag != 0) {
-            status = flag;
+        if (sum_cnt < 0) {
+            status = -5 /*BM_ERR_TIMEOUT*/;
             break;
         }
         if (leader) {
@@ -624,6 +626,7 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
         __syncthreads();
         for (int w = t; w < words; w += T) srv[w] = 0u;
         for (int w = t; w < (int)((lay.cm - lay.rcl) >> 2); w += T) rcl[w] = 0u;
+        if (leader && bmd::globaltimer() > deadline) sm.mine.flag = -5 /*BM_ERR_TIMEOUT*/;
         end_step(true);
 #ifdef BM_CHECKED
         check_matching();
@@ -702,7 +705,8 @@ __global__ void __launch_bounds__(T, 1) k_solo(Params p, SoloArgs a, long long n
 // more than GREEDY_LIGHT rows a warp each from the block's list.  Adds to the
 // installed matching; |M| goes to the control block and the host's copy.
 template <int C, int T>
-__global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* __restrict__ rdeg, Ctl* h_ctl, int check_err) {
+__global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* __restrict__ rdeg, Ctl* h_ctl, int check_err,
+                                                     int crowded) {
     using namespace bmd;
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ int s_card, s_long;
@@ -715,7 +719,9 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     // an invalid CSR is not read (the same in every block: nothing writes the word then)
     const int err = check_err ? ld_volatile(&p.ctl->err) : 0;
     if (err != 0) return;
+#ifdef BM_CHECKED
     if (!check_err && rank == 0 && t == 0) p.ctl->err = 0;
+#endif
     if (t == 0) s_card = s_long = 0;
     __syncthreads();
     int n = 0;
@@ -733,7 +739,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     auto state_of = [&](int r) { return idx_ok(p, r, nr) ? (int)dld32(state_at(r)) : GREEDY_TAKEN; };
     auto take = [&](int r, int seen) { return dcas(state_at(r), seen, GREEDY_TAKEN) == seen; };
     const int limit[4] = {0, 2, 8, GREEDY_LIGHT};
-    const bool crowded = greedy_crowded(nr, __ldg(&p.col_ptr[nc])), any = crowded && nc > 2LL * nr;
+    const bool any = crowded && nc > 2LL * nr;
 #pragma unroll 1
     for (int k = 0; k < 3; ++k) {
         for (unsigned k0 = warp; k0 < (1u << bits); k0 += T / 32) {
@@ -758,7 +764,7 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
         const int c = longs[k];
         if (p.cmatch[c] != -1) continue;
         const int beg = __ldg(&p.col_ptr[c]), deg = __ldg(&p.col_ptr[c + 1]) - beg;
-        const int r = greedy_warp(p.row_idx + beg, deg, c, hash32((unsigned)c), crowded, state_of, take);
+        const int r = greedy_warp(p.row_idx + beg, deg, c, hash32((unsigned)c), crowded != 0, state_of, take);
         if (r >= 0 && lane == 0) {
             p.rmatch[r] = c;
             p.cmatch[c] = r;
@@ -771,7 +777,9 @@ __global__ void __launch_bounds__(T, 1) k_solo_greedy(Params p, const int32_t* _
     if (rank == 0 && t == 0) {
         Ctl c{};
         c.card = s_card;
-        c.err = ld_volatile(&p.ctl->err);  // (range-checked build)
+#ifdef BM_CHECKED
+        c.err = ld_volatile(&p.ctl->err);
+#endif
         *p.ctl = c;
         *h_ctl = c;
     }

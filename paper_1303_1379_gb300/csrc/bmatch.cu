@@ -1337,7 +1337,8 @@ int32_t run_solo_greedy(bm_ctx* ctx, bool check_err) {
     const int C = solo_cluster(ctx);
     const size_t smem = 128 * ((((size_t)ctx->nr + 31) / 32 + C - 1) / C);
     BM_CUDA(ctx, launch_cluster(C == 1 ? bms1::k_solo_greedy<1, bms1::SOLO_T1> : bms1::k_solo_greedy<kSoloBlocks, bms1::SOLO_T>, C, smem, ctx->stream,
-                          make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl, check_err ? 1 : 0));
+                          make_params(ctx, false), (const int32_t*)ctx->rdeg, ctx->h_ctl, check_err ? 1 : 0,
+                          bmd::greedy_crowded(ctx->nr, ctx->nnz) ? 1 : 0));
     return BM_OK;
 }
 
