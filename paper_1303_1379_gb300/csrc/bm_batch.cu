@@ -296,22 +296,25 @@ double launch_estimate(const std::vector<int64_t>& edges, int slots, double slop
 
 // Whether a batch whose caller leaves the launch to the library gets one block of 1,024 threads an SM (else two of
 // 512).  The wider block is the faster one for a graph by itself, by the more the larger the graph, and for the
-// smallest no faster; but there are half as many.  So both launches are estimated from the graphs' entries: a graph
-// takes about as long as 16,000 entries more than it has (a few dozen barriers), and 1.8 times as long per entry on
-// the narrower of two blocks an SM (2.3 times with the deterministic option and more data than L2 holds, about 28
-// bytes a row and a column and 4 an entry).  One GB300, ms at 512 / 1,024 threads, default and deterministic:
-// graphs of 100 to 50,000 rows, 48 of them 1.31 / 0.97, 3.97 / 2.38; 512 2.17 / 1.40, 6.7 / 4.8; 2,048 3.0 / 2.7,
-// 15.2 / 11.7; 4,096 4.86 / 5.00; equal graphs of 1,000 rows, 152 of them 0.168 / 0.167, 0.48 / 0.42; 200 0.169 /
-// 0.236, 0.46 / 0.62; 400 0.23 / 0.32, 0.72 / 0.91; of 20,000 rows, 100 0.92 / 0.55, 3.1 / 2.1; 200 1.08 / 1.03, 5.0
-// / 4.5; 400 1.9 / 1.55, 10.4 / 7.6; one of 50,000 rows and 1,000 of 200 2.0 / 1.4, 4.9 / 3.5, and 8,000 of 200 2.1 /
-// 2.6, 6.0 / 7.0; 300 meshes of 60 x 60 0.72 / 0.88, 3.5 / 5.7.
+// smallest no faster; but there are half as many.  So a batch of less than 2 x SMs times the largest graph's entries
+// gets it, a larger one, which keeps every block busy to the end, does not: graphs of 100 to 50,000 rows, ms at 512 /
+// 1,024 threads, default and deterministic: 48 of them 1.31 / 0.97, 3.97 / 2.38; 512 2.17 / 1.40, 6.7 / 4.8; 2,048
+// 3.0 / 2.7, 15.2 / 11.7; 2,774, of which one takes 4.8 ms on the wider block, 7.45 / 4.83; 4,096 4.86 / 5.00.
+// Unless the graphs' entries say clearly that the other launch is shorter (the slowest graphs take up to three times
+// as long as others of their size): a graph is estimated at 16,000 entries more than it has (a few dozen barriers)
+// and 1.8 times as long per entry on one of two blocks an SM (2.3 times with the deterministic option and more data
+// than L2 holds, about 28 bytes a row and a column and 4 an entry).  Equal graphs of 1,000 rows, 152 of them 0.168 /
+// 0.167, 0.48 / 0.42; 200 0.169 / 0.236, 0.46 / 0.62; 300 meshes of 60 x 60 0.72 / 0.88, 3.5 / 5.7; equal graphs of
+// 20,000 rows, 200 1.08 / 1.03, 5.0 / 4.5; 400 1.9 / 1.55, 10.4 / 7.6.
 bool wide_blocks(const bm_batch* b) {
     const int64_t n = (int64_t)b->edges.size();
     if (n <= b->num_sms) return n > 0;
+    const bool few = b->total_edges < 2 * (int64_t)b->num_sms * b->edges[0];
     const double at_once = std::min(1.0, 2.0 * b->num_sms / (double)n);  // part of the batch on the chip
     const bool spills = at_once * (28.0 * (double)(b->total_rows + b->total_cols) + 4.0 * (double)b->total_edges) > b->l2_bytes;
-    return launch_estimate(b->edges, b->num_sms, 1.0) <=
-           launch_estimate(b->edges, 2 * b->num_sms, b->opt.deterministic && spills ? 2.3 : 1.8);
+    const double wide = launch_estimate(b->edges, b->num_sms, 1.0);
+    const double narrow = launch_estimate(b->edges, 2 * b->num_sms, b->opt.deterministic && spills ? 2.3 : 1.8);
+    return few ? wide < 1.25 * narrow : wide < 0.95 * narrow;
 }
 
 // The entry counts are read by the cheap matching of the default routine (block_greedy_sb).

@@ -95,7 +95,7 @@ def test_batch_counts_rows_when_an_option_comes_to_read_them(first):
     # rows x graphs; one block of 1,024 threads an SM holds 152 graphs at once, two of 512 hold 304
     ([(200, 152)], 0, 1024), ([(200, 153)], 0, 512), ([(200, 303)], 1, 512), ([(1000, 200)], 0, 512),
     ([(1000, 200)], 1, 512), ([(10000, 1), (200, 600)], 0, 1024), ([(40000, 1), (200, 300)], 0, 1024),
-    ([(40000, 8), (200, 300)], 1, 1024), ([(3000, 20), (100, 280)], 0, 512), ([(20000, 310)], 1, 1024), ([(20000, 310)], 0, 1024),
+    ([(40000, 8), (200, 300)], 1, 1024), ([(3000, 20), (100, 280)], 0, 1024), ([(3000, 20), (2500, 280)], 0, 512), ([(20000, 310)], 1, 1024), ([(20000, 310)], 0, 1024),
 ], ids=str)
 def test_batch_default_geometry_by_the_longest_wait(sizes, det, block):
     pool = {nr: synth.uniform_graph(nr, nr + nr // 20, 7, seed=nr) for nr, _ in sizes}
