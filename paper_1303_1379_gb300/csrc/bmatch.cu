@@ -841,7 +841,7 @@ struct bm_ctx {
     int32_t* rvis = nullptr;     // per-row claim stamps of the persistent kernel
     int32_t* rdeg = nullptr;     // per-row number of entries, for the cheap matching (ensure_rdeg)
     bool rdeg_ready = false;     // ... they are those of the present CSR
-    bool rdeg_read = false;      // ... and a cheap matching has read them
+    bool rdeg_read = true;       // ... and a cheap matching has read them (before the first CSR: expected)
     int2* crec = nullptr;        // per-column (parent column, matched row) of the last search
     long long stamp_next = 0;    // every stamp in rvis is below stamp_next + 1
     int32_t* profile = nullptr;  // kProfileCap phases x 4
@@ -1085,9 +1085,9 @@ int32_t validate_csr_async(bm_ctx* ctx, bool count) {
     return BM_OK;
 }
 
-// The rows' entry counts, which only the cheap matching of the default option reads: counted when it is first
-// called on a CSR (checked before), not with every CSR that arrives.  An upload makes them with its check, in one
-// pass, if those of the CSR before were read (200 k columns: 39 us together, 11 + 38 us apart).
+// The rows' entry counts, which only the cheap matching of the default option reads.  They are made with the check of
+// a context's first CSR, in one pass over the entries, and with that of an upload if those of the CSR before were read
+// (200 k columns of 12: 39 us together, 11 + 38 us apart); otherwise here, when the cheap matching is called after all.
 int32_t ensure_rdeg(bm_ctx* ctx) {
     ctx->rdeg_read = true;
     if (ctx->rdeg_ready) return BM_OK;
@@ -1521,7 +1521,7 @@ int32_t bm_create(int32_t n_rows, int32_t n_cols, int64_t nnz, const int32_t* co
         return BM_ERR_CUDA;
     }
     if (!own) {
-        rc = validate_csr_async(ctx, false);
+        rc = validate_csr_async(ctx, !o.deterministic);
         if (!rc) rc = sync_ctl(ctx);
         if (!rc && ctx->h_ctl->err) rc = ctx->h_ctl->err;
         if (rc) { bm_destroy(ctx); return rc; }
